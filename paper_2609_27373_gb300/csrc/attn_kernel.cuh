@@ -1,4 +1,5 @@
-// Causal flash attention on tcgen05 tensor cores, in three variants:
+// Causal flash attention on tcgen05 tensor cores, for launches with few query
+// tiles per SM (attn_duo.cuh has the kernel for the others), in three variants:
 //   kDense      O = softmax(Q K^T * scale + M) V                  (Eq. 2)
 //   kDenseMass  the same, plus the block attention mass of the step (Eq. 5)
 //               accumulated into blockmass

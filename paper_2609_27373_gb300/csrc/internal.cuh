@@ -27,6 +27,9 @@ __host__ __device__ constexpr size_t scratch_floats_per_cta(int n_tiles, int sub
 constexpr int kStatusTimeout = 1;
 constexpr int kStatusBadSupport = 2;
 
+// How the two streams of attn_duo_kernel take query tiles (attn_duo.cuh).
+enum AttnPair : int { kPairNone = 0, kPairHeads = 1, kPairTiles = 2 };
+
 struct AttnParams {
   int batch, seqlen, n_heads, n_kv_heads, group;
   int n_qtiles;   // ceil(seqlen / 128): 128-row query tiles
@@ -43,6 +46,10 @@ struct AttnParams {
   float* scratch;         // kDenseMass: scratch_floats_per_cta(n_blocks) floats per CTA
   int* status;
   unsigned long long wait_ns;  // limit of each bounded wait on the main path (kWaitLimitNs by default)
+  // attn_duo_kernel: the pairing, and its units (virtual heads and query
+  // tiles, see decode_duo).
+  int pair, v_heads, v_qtiles, v_units, v_group_heads;
+  int o_align32;  // O is 32-byte aligned
 };
 
 struct AttnLaunch {
@@ -57,6 +64,11 @@ struct AttnLaunch {
 cudaError_t launch_attn_d64(int block, int mode, const AttnLaunch& L);
 cudaError_t launch_attn_d96(int block, int mode, const AttnLaunch& L);
 cudaError_t launch_attn_d128(int block, int mode, const AttnLaunch& L);
+
+// Defined in duo_d64.cu / duo_d96.cu / duo_d128.cu.
+cudaError_t launch_duo_d64(int block, int mode, const AttnLaunch& L);
+cudaError_t launch_duo_d96(int block, int mode, const AttnLaunch& L);
+cudaError_t launch_duo_d128(int block, int mode, const AttnLaunch& L);
 
 struct SelectParams {
   int batch, n_heads, n_kv_heads, group, n_blocks;

@@ -134,6 +134,41 @@ bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Whether a launch runs on attn_duo_kernel (two query tiles in flight per CTA)
+// rather than attn_kernel (both softmax warpgroups on one), and its pairing.
+// With few units a CTA of the former has no second one to overlap with the
+// first, and a unit alone takes longer there.  Measured (us, attn_kernel /
+// attn_duo_kernel; d = head dim):
+//   dense: 256 units (2K, 16 heads, d 128) 20.2 / 28.9, 384 (4K, 12 heads) 47.5 / 52.0,
+//     512 (4K, 16 heads) 57.3 / 52.8, 1024 (4K, 32 heads) 119 / 105;
+//   sparse, block 128, d 128: 384 27.6 / 29.9, 512 (4K) 32.7 / 33.4, 512 (8K) 42.0 /
+//     40.4, 1024 (8K) 74.3 / 71.1, 1024 (4K, 32 heads) 63 / 58; d 96: 768 44.2 / 43.0;
+//   sparse, block 32 or 64, or d 64: 192 19.9 / 26.6, 512 (d 64, block 64) 37.2 / 29.0,
+//     512 (d 128, block 64) 62.7 / 55.6, 512 (d 64, block 64, 512 tokens) 19.7 / 15.3.
+// The line depends on the shape alone, not on the variant: sparse attention
+// over every block and dense attention run on the same kernel and give the
+// same bits.
+bool choose_duo(int mode, const wise_shape_t* sh, int sm_count, AttnParams& p) {
+  if (p.n_qtiles > 256) return false;  // the staged tile masks hold 256 key tiles
+  const bool wide = sh->block == 128 && sh->head_dim > 64;
+  if (p.n_units < (wide ? 4 : 3) * sm_count) return false;
+  p.pair = kPairNone;
+  p.v_heads = p.n_heads;
+  p.v_qtiles = p.n_qtiles;
+  p.v_group_heads = p.group_heads;
+  if (p.group % 2 == 0) {
+    // Two heads of a kv-head group read the same K, V and support.
+    p.pair = kPairHeads;
+    p.v_heads = p.n_heads / 2;
+    p.v_group_heads = p.group_heads / 2;
+  } else if (mode != kSparse) {
+    p.pair = kPairTiles;
+    p.v_qtiles = (p.n_qtiles + 1) / 2;
+  }
+  p.v_units = p.batch * p.v_heads * p.v_qtiles;
+  return true;
+}
+
 }  // namespace
 
 int launch_attention(const wise_shape_t* sh, const void* Q, const void* K, const void* V, void* O, int mode,
@@ -218,6 +253,16 @@ int launch_attention(const wise_shape_t* sh, const void* Q, const void* K, const
     }
   }
   cudaError_t e;
+  if (choose_duo(mode, sh, ds->sm_count, p)) {
+    p.o_align32 = aligned(O, 32);
+    L.grid = std::min(p.v_units, ds->sm_count);
+    switch (sh->head_dim) {
+      case 64: e = launch_duo_d64(sh->block, mode, L); break;
+      case 96: e = launch_duo_d96(sh->block, mode, L); break;
+      default: e = launch_duo_d128(sh->block, mode, L); break;
+    }
+    return e == cudaSuccess ? WISE_OK : WISE_ERR_CUDA;
+  }
   switch (sh->head_dim) {
     case 64: e = launch_attn_d64(sh->block, mode, L); break;
     case 96: e = launch_attn_d96(sh->block, mode, L); break;
