@@ -1,30 +1,56 @@
-// Support selection (Eq. 6, single-pass form over accumulated block mass).
+// Support selection (Eq. 6, single-pass form over accumulated block mass) and
+// the working sets of the paper's own form.
 //
 // One warp per (batch, kv-head, query block) row.  Lane l owns key blocks
 // l, l + 32, ... (KPL of them).  Masses of the kv-head group's query heads are
 // pooled in exact 64-bit fixed point, the forced sink/local blocks are marked,
-// and the remaining admissible blocks are taken one at a time in rank order
-// (pooled mass descending, block index ascending) by a warp-wide argmax over
-// shuffles, until top-k is reached or the kept mass covers eta of the row's
-// admissible mass (cum * 65536 >= eta16 * total, compared in 128 bits), never
-// beyond `cap`.  The chosen set is written in ascending order with ballots and
-// prefix popcounts, padded with -1.
+// and the remaining admissible blocks are taken in rank order (pooled mass
+// descending, block index ascending) until the rule is met: top-k reached, or
+// the kept mass covering eta of the row's admissible mass
+// (cum * 65536 >= eta16 * total, compared in 128 bits), never beyond `cap`.
+// The chosen set is written in ascending order with ballots and prefix
+// popcounts, padded with -1.
+//
+// Bound: latency and instruction issue (the masses of a 32K launch are 4 MB).
+// The fixed-point conversion is integer arithmetic, not double precision, whose
+// rate on this chip is 1/64 of single precision's, and reductions use the warp
+// reduction instructions.  Ranking (take_ranked) depends on the row: up to 32
+// blocks are compared all with all, few picks are taken one by one, and many by
+// a binary search for the mass of the last pick.  Measured back to back in a
+// graph (us, with double precision, one-by-one picks and shuffles / here): 32K,
+// 4 heads per kv head, top 12: 22.6 / 12.8; coverage up to 32 of 128 blocks 32.8 /
+// 18.0; working sets of 4 steps: 4K 40 / 8.6, 16K (128 blocks) 316 / 58, 32K (5
+// steps) 734 / 84.
 #include <limits.h>
 
 #include "internal.cuh"
 
 namespace wise {
 
+// floor(min(x, 4096) * 2^32); negative, zero and NaN masses count as zero.
 __device__ __forceinline__ uint64_t mass_units(float x) {
-  if (!(x > 0.0f)) return 0ull;  // negative, zero and NaN masses count as zero
-  x = fminf(x, 4096.0f);
-  return __double2ull_rz(floor(static_cast<double>(x) * 4294967296.0));
+  if (!(x > 0.0f)) return 0ull;
+  const uint32_t bits = __float_as_uint(fminf(x, 4096.0f));
+  const int shift = (int)(bits >> 23) - 118;  // x = m * 2^(e - 150)
+  const uint64_t m = (bits & 0x7FFFFFu) | 0x800000u;
+  // Below 2^-32 (denormals among them) the result is 0: m < 2^24.
+  return shift >= 0 ? m << shift : shift > -24 ? m >> -shift : 0ull;
 }
 
+// Sum over the warp of values below 2^59 (the total below 2^64): 26-bit limbs,
+// whose sums of 32 fit a 32-bit reduction.
 __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  return v;
+  constexpr uint32_t kLimb = (1u << 26) - 1u;
+  const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)v & kLimb);
+  const uint32_t s1 = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 26) & kLimb);
+  const uint32_t s2 = __reduce_add_sync(0xffffffffu, (uint32_t)(v >> 52));
+  return (uint64_t)s0 + ((uint64_t)s1 << 26) + ((uint64_t)s2 << 52);
+}
+
+__device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
+  const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32));
+  const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
+  return ((uint64_t)hi << 32) | lo;
 }
 
 // cum * 65536 < eta16 * total, exactly.
@@ -32,6 +58,135 @@ __device__ __forceinline__ bool below_threshold(uint64_t cum, uint64_t eta16, ui
   const uint64_t lhs_hi = cum >> 48, lhs_lo = cum << 16;
   const uint64_t rhs_hi = __umul64hi(eta16, total), rhs_lo = eta16 * total;
   return lhs_hi < rhs_hi || (lhs_hi == rhs_hi && lhs_lo < rhs_lo);
+}
+
+// Adds candidates in rank order to `chosen` until done(kept mass, number
+// added), which stays true once it is true; `cum` is the mass kept before, and
+// `most` an upper bound on the number added.  Bit i of cand / chosen is block
+// lane + 32 i.
+template <int KPL, class Done>
+__device__ __forceinline__ void take_ranked(const uint64_t (&U)[KPL], uint32_t cand, uint32_t& chosen, uint64_t cum,
+                                            int most, int lane, Done done) {
+  if (done(cum, 0)) return;
+  if constexpr (KPL == 1) {
+    // Lane l's block is taken unless the blocks ranked before it (mass and
+    // number summed over all of them) already suffice.
+    uint64_t before = 0;
+    int rank = 0;
+    const uint32_t all = __ballot_sync(0xffffffffu, cand != 0u);
+    const uint64_t mine = U[0];
+#pragma unroll 8
+    for (int o = 0; o < 32; ++o) {
+      const uint64_t u = __shfl_sync(0xffffffffu, mine, o);
+      const bool ahead = ((all >> o) & 1u) && (u > mine || (u == mine && o < lane));
+      before += ahead ? u : 0ull;
+      rank += ahead;
+    }
+    if (cand && !done(cum + before, rank)) chosen |= 1u;
+  } else {
+    int added = 0;
+    if (most > 16) {
+      // The largest T such that the blocks of mass >= T suffice, bit by bit.
+      uint64_t top = 0, part = 0;
+#pragma unroll
+      for (int i = 0; i < KPL; ++i) {
+        if ((cand >> i) & 1u) {
+          top = max(top, U[i]);
+          part += U[i];
+        }
+      }
+      if (!done(cum + warp_sum_u64(part), __reduce_add_sync(0xffffffffu, __popc(cand)))) {
+        chosen |= cand;  // all of them do not suffice
+        return;
+      }
+      top = warp_max_u64(top);
+      uint64_t T = 0;
+      for (int bit = 63 - __clzll((long long)(top | 1ull)); bit >= 0; --bit) {
+        const uint64_t t = T | (1ull << bit);
+        uint64_t s = 0;
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < KPL; ++i) {
+          const bool in = ((cand >> i) & 1u) && U[i] >= t;
+          s += in ? U[i] : 0ull;
+          n += in;
+        }
+        if (done(cum + warp_sum_u64(s), __reduce_add_sync(0xffffffffu, n))) T = t;
+      }
+      // Every block above T; those of mass T one by one below.
+      uint64_t s = 0;
+      uint32_t above = 0, equal = 0;
+#pragma unroll
+      for (int i = 0; i < KPL; ++i) {
+        if (!((cand >> i) & 1u)) continue;
+        if (U[i] > T) {
+          above |= 1u << i;
+          s += U[i];
+        } else if (U[i] == T) {
+          equal |= 1u << i;
+        }
+      }
+      chosen |= above;
+      cum += warp_sum_u64(s);
+      added = __reduce_add_sync(0xffffffffu, __popc(above));
+      cand = equal;
+    }
+    // One at a time: the largest mass, then the lowest block.
+    while (!done(cum, added)) {
+      uint64_t best_u = 0;
+      int best_kb = INT_MAX;
+#pragma unroll
+      for (int i = 0; i < KPL; ++i) {
+        if (((cand >> i) & 1u) && (best_kb == INT_MAX || U[i] > best_u)) {
+          best_u = U[i];
+          best_kb = lane + 32 * i;
+        }
+      }
+      const uint64_t u = warp_max_u64(best_u);
+      const int kb = (int)__reduce_min_sync(0xffffffffu, best_u == u ? (uint32_t)best_kb : (uint32_t)INT_MAX);
+      if (kb == INT_MAX) return;  // no candidate left
+      if ((kb & 31) == lane) {
+        cand &= ~(1u << (kb >> 5));
+        chosen |= 1u << (kb >> 5);
+      }
+      cum += u;
+      ++added;
+    }
+  }
+}
+
+// Pooled masses of this lane's blocks in one row set of masses
+// [batch][n_heads][nb][nb].
+template <int KPL>
+__device__ __forceinline__ void pool_masses(const float* masses, int n_heads, int group, int nb, int b, int g, int q,
+                                            int lane, uint64_t (&U)[KPL]) {
+  const float* row = masses + (((size_t)b * n_heads + (size_t)g * group) * nb + q) * nb;
+  const size_t head = (size_t)nb * nb;
+#pragma unroll
+  for (int i = 0; i < KPL; ++i) U[i] = 0;
+#pragma unroll 4
+  for (int h = 0; h < group; ++h) {
+#pragma unroll
+    for (int i = 0; i < KPL; ++i) {
+      const int kb = lane + 32 * i;
+      if (kb <= q) U[i] += mass_units(__ldg(row + h * head + kb));
+    }
+  }
+}
+
+// Writes the chosen blocks of a row in ascending order, -1 padded, and their
+// number.
+template <int KPL>
+__device__ __forceinline__ void write_row(uint32_t chosen, int32_t* out, int cap, int32_t* count, int lane) {
+  int n = 0;
+#pragma unroll
+  for (int i = 0; i < KPL; ++i) {
+    const uint32_t ball = __ballot_sync(0xffffffffu, (chosen >> i) & 1u);
+    if ((chosen >> i) & 1u) out[n + __popc(ball & ((1u << lane) - 1u))] = lane + 32 * i;
+    n += __popc(ball);
+  }
+  for (int pos = n + lane; pos < cap; pos += 32) out[pos] = -1;
+  if (lane == 0) *count = n;
 }
 
 template <int KPL>
@@ -46,15 +201,13 @@ __global__ void __launch_bounds__(256) select_kernel(const SelectParams p) {
   const int b = (int)(row / ((long)nb * p.n_kv_heads));
 
   uint64_t U[KPL];
+  pool_masses(p.blockmass, p.n_heads, p.group, nb, b, g, q, lane, U);
   uint32_t cand = 0, chosen = 0;  // bit i <-> block lane + 32 i
   uint64_t total_part = 0, cum_part = 0;
 #pragma unroll
   for (int i = 0; i < KPL; ++i) {
     const int kb = lane + 32 * i;
-    U[i] = 0;
     if (kb <= q) {
-      for (int h = g * p.group; h < (g + 1) * p.group; ++h)
-        U[i] += mass_units(__ldg(p.blockmass + (((size_t)b * p.n_heads + h) * nb + q) * nb + kb));
       total_part += U[i];
       const bool forced = kb < p.n_sink || kb > q - p.n_local;
       if (forced) {
@@ -66,54 +219,14 @@ __global__ void __launch_bounds__(256) select_kernel(const SelectParams p) {
     }
   }
   const uint64_t total = warp_sum_u64(total_part);
-  uint64_t cum = warp_sum_u64(cum_part);
-  int n = 0;
-#pragma unroll
-  for (int i = 0; i < KPL; ++i) n += __popc(__ballot_sync(0xffffffffu, (chosen >> i) & 1u));
-
-  const int budget = (p.mode == 0) ? min(p.topk, p.cap - n) : p.cap - n;
-  for (int t = 0; t < budget; ++t) {
-    if (p.mode != 0 && !below_threshold(cum, p.eta16, total)) break;
-    // Best candidate of this lane: larger mass first, then lower block.
-    uint64_t best_u = 0;
-    int best_kb = INT_MAX;
-#pragma unroll
-    for (int i = 0; i < KPL; ++i) {
-      if (((cand >> i) & 1u) && (best_kb == INT_MAX || U[i] > best_u)) {
-        best_u = U[i];
-        best_kb = lane + 32 * i;
-      }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const uint64_t ou = __shfl_xor_sync(0xffffffffu, best_u, off);
-      const int okb = __shfl_xor_sync(0xffffffffu, best_kb, off);
-      const bool take = (okb != INT_MAX) && (best_kb == INT_MAX || ou > best_u || (ou == best_u && okb < best_kb));
-      if (take) {
-        best_u = ou;
-        best_kb = okb;
-      }
-    }
-    if (best_kb == INT_MAX) break;  // no candidate left
-    if ((best_kb & 31) == lane) {
-      const uint32_t bit = 1u << (best_kb >> 5);
-      cand &= ~bit;
-      chosen |= bit;
-    }
-    cum += best_u;
-    ++n;
-  }
-
-  int32_t* out = p.idx + row * p.cap;
-  int base = 0;
-#pragma unroll
-  for (int i = 0; i < KPL; ++i) {
-    const uint32_t ball = __ballot_sync(0xffffffffu, (chosen >> i) & 1u);
-    if ((chosen >> i) & 1u) out[base + __popc(ball & ((1u << lane) - 1u))] = lane + 32 * i;
-    base += __popc(ball);
-  }
-  for (int pos = n + lane; pos < p.cap; pos += 32) out[pos] = -1;
-  if (lane == 0) p.counts[row] = n;
+  const uint64_t cum = warp_sum_u64(cum_part);
+  const int n_forced = __reduce_add_sync(0xffffffffu, __popc(chosen));
+  const int budget = (p.mode == 0) ? min(p.topk, p.cap - n_forced) : p.cap - n_forced;
+  const bool coverage = p.mode != 0;
+  take_ranked(U, cand, chosen, cum, budget, lane, [&](uint64_t c, int n) {
+    return n >= budget || (coverage && !below_threshold(c, p.eta16, total));
+  });
+  write_row<KPL>(chosen, p.idx + row * p.cap, p.cap, p.counts + row, lane);
 }
 
 template <int KPL>
@@ -143,66 +256,6 @@ cudaError_t launch_select(const SelectParams& p, cudaStream_t stream) {
 // 2 mass matched, 3 size matched (first step's ranking against a reference
 // working set).  Forced sink/local blocks belong to every set.
 
-// Warp-wide best remaining candidate: larger mass first, then lower block.
-template <int KPL>
-__device__ __forceinline__ int ws_argmax(const uint64_t (&U)[KPL], uint32_t cand, int lane, uint64_t& best_u) {
-  best_u = 0;
-  int best_kb = INT_MAX;
-#pragma unroll
-  for (int i = 0; i < KPL; ++i) {
-    if (((cand >> i) & 1u) && (best_kb == INT_MAX || U[i] > best_u)) {
-      best_u = U[i];
-      best_kb = lane + 32 * i;
-    }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const uint64_t ou = __shfl_xor_sync(0xffffffffu, best_u, off);
-    const int okb = __shfl_xor_sync(0xffffffffu, best_kb, off);
-    const bool take = (okb != INT_MAX) && (best_kb == INT_MAX || ou > best_u || (ou == best_u && okb < best_kb));
-    if (take) {
-      best_u = ou;
-      best_kb = okb;
-    }
-  }
-  return best_kb;
-}
-
-// Pooled fixed-point masses of one step for this lane's blocks.
-template <int KPL>
-__device__ __forceinline__ void ws_pool(const WorkingSetParams& p, int step, int b, int g, int q, int lane,
-                                        uint64_t (&U)[KPL]) {
-  const int nb = p.n_blocks;
-  const float* m = p.masses + (size_t)step * p.batch * p.n_heads * nb * nb;
-#pragma unroll
-  for (int i = 0; i < KPL; ++i) {
-    const int kb = lane + 32 * i;
-    U[i] = 0;
-    if (kb <= q)
-      for (int h = g * p.group; h < (g + 1) * p.group; ++h)
-        U[i] += mass_units(__ldg(m + (((size_t)b * p.n_heads + h) * nb + q) * nb + kb));
-  }
-}
-
-// Adds candidates in rank order to `chosen` (mass cum) until stop(cum) or
-// `budget` additions or no candidate is left.
-template <int KPL, class Stop>
-__device__ __forceinline__ void ws_take(const uint64_t (&U)[KPL], uint32_t& cand, uint32_t& chosen, uint64_t& cum,
-                                        int budget, int lane, Stop stop) {
-  for (int t = 0; t < budget; ++t) {
-    if (stop(cum)) break;
-    uint64_t best_u;
-    const int best_kb = ws_argmax(U, cand, lane, best_u);
-    if (best_kb == INT_MAX) break;
-    if ((best_kb & 31) == lane) {
-      const uint32_t bit = 1u << (best_kb >> 5);
-      cand &= ~bit;
-      chosen |= bit;
-    }
-    cum += best_u;
-  }
-}
-
 template <int KPL>
 __global__ void __launch_bounds__(256) working_set_kernel(const WorkingSetParams p) {
   const long row = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -224,11 +277,12 @@ __global__ void __launch_bounds__(256) working_set_kernel(const WorkingSetParams
     }
   }
   uint64_t U[KPL];
+  const size_t step_size = (size_t)p.batch * p.n_heads * nb * nb;
   uint32_t result = forced;
   if (p.mode <= 1) {
     // Union over the steps of each step's eta coverage set (one step: static).
     for (int st = 0; st < p.n_steps; ++st) {
-      ws_pool(p, st, b, g, q, lane, U);
+      pool_masses(p.masses + (size_t)st * step_size, p.n_heads, p.group, nb, b, g, q, lane, U);
       uint64_t total_part = 0, cum_part = 0;
 #pragma unroll
       for (int i = 0; i < KPL; ++i) {
@@ -236,15 +290,14 @@ __global__ void __launch_bounds__(256) working_set_kernel(const WorkingSetParams
         if ((forced >> i) & 1u) cum_part += U[i];
       }
       const uint64_t total = warp_sum_u64(total_part);
-      uint64_t cum = warp_sum_u64(cum_part);
-      uint32_t cand = admissible & ~forced, chosen = forced;
-      ws_take(U, cand, chosen, cum, nb, lane,
-              [&](uint64_t c) { return !below_threshold(c, p.eta16, total); });
+      uint32_t chosen = forced;
+      take_ranked(U, admissible & ~forced, chosen, warp_sum_u64(cum_part), nb, lane,
+                  [&](uint64_t c, int) { return !below_threshold(c, p.eta16, total); });
       result |= chosen;
     }
   } else {
     // The reference working set of this row: its size and its first-step mass.
-    ws_pool(p, 0, b, g, q, lane, U);
+    pool_masses(p.masses, p.n_heads, p.group, nb, b, g, q, lane, U);
     const int32_t* ref = p.ref_idx + row * p.ref_cap;
     int n_ref = __ldg(p.ref_counts + row);
     int bad = 0;
@@ -276,28 +329,16 @@ __global__ void __launch_bounds__(256) working_set_kernel(const WorkingSetParams
       }
     }
     const uint64_t target = warp_sum_u64(ref_part);
-    uint64_t cum = warp_sum_u64(cum_part);
-    int n_forced = n_forced_part;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) n_forced += __shfl_xor_sync(0xffffffffu, n_forced, off);
-    uint32_t cand = admissible & ~forced, chosen = forced;
+    const uint64_t cum = warp_sum_u64(cum_part);
+    const int k_more = k_ref - __reduce_add_sync(0xffffffffu, n_forced_part);
+    uint32_t chosen = forced;
     if (p.mode == 2)
-      ws_take(U, cand, chosen, cum, nb, lane, [&](uint64_t c) { return c >= target; });
+      take_ranked(U, admissible & ~forced, chosen, cum, nb, lane, [&](uint64_t c, int) { return c >= target; });
     else
-      ws_take(U, cand, chosen, cum, k_ref - n_forced, lane, [](uint64_t) { return false; });
+      take_ranked(U, admissible & ~forced, chosen, cum, k_more, lane, [&](uint64_t, int n) { return n >= k_more; });
     result = chosen;
   }
-
-  int32_t* out = p.idx + row * p.cap;
-  int base = 0;
-#pragma unroll
-  for (int i = 0; i < KPL; ++i) {
-    const uint32_t ball = __ballot_sync(0xffffffffu, (result >> i) & 1u);
-    if ((result >> i) & 1u) out[base + __popc(ball & ((1u << lane) - 1u))] = lane + 32 * i;
-    base += __popc(ball);
-  }
-  for (int pos = base + lane; pos < p.cap; pos += 32) out[pos] = -1;
-  if (lane == 0) p.counts[row] = base;
+  write_row<KPL>(result, p.idx + row * p.cap, p.cap, p.counts + row, lane);
 }
 
 template <int KPL>
