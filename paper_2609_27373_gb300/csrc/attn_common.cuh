@@ -9,6 +9,8 @@
 #include <limits.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "internal.cuh"
 #include "ptx.cuh"
 
@@ -306,6 +308,40 @@ template <int BLK>
 __device__ __forceinline__ void load_s_row(uint32_t addr, float (&s)[kTileN], uint32_t sub, int lim) {
   tmem_load_row<kTileN>(addr, s);
   mask_s_row<BLK>(s, sub, lim);
+}
+
+// Launches an attention kernel with programmatic stream serialization: the
+// grid may be scheduled while the previous kernel of the stream finishes (see
+// griddep_wait in the kernels).  The kernel's shared-memory limit is raised on
+// its first launch on each device (the call costs a launch about 0.5 us), and
+// again if a launch fails, as after a reset of the device.
+template <auto kKernel, class... Args>
+cudaError_t launch_dependent(int grid, int threads, int smem, cudaStream_t stream, const Args&... args) {
+  static std::atomic<uint64_t> raised{0};  // bit per device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+  if (raised.load(std::memory_order_relaxed) & bit) {
+    if (cudaLaunchKernelEx(&cfg, kKernel, args...) == cudaSuccess) return cudaGetLastError();
+    cudaGetLastError();
+  }
+  e = cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  raised.fetch_or(bit, std::memory_order_relaxed);
+  e = cudaLaunchKernelEx(&cfg, kKernel, args...);
+  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
 }
 
 }  // namespace wise

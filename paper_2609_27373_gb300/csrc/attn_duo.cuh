@@ -1153,22 +1153,7 @@ __global__ void __launch_bounds__(512, 1)
 template <int D, int BLK, int MODE, bool kPaired>
 cudaError_t launch_duo_instance(const AttnLaunch& L) {
   using C = DuoCfg<D, kPaired>;
-  auto kern = attn_duo_kernel<D, BLK, MODE, kPaired>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(L.grid);
-  cfg.blockDim = dim3(C::kThreads);
-  cfg.dynamicSmemBytes = C::kSmem;
-  cfg.stream = L.stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, L.mapQ, L.mapK, L.mapV, L.p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_dependent<attn_duo_kernel<D, BLK, MODE, kPaired>>(L.grid, C::kThreads, C::kSmem, L.stream, L.mapQ, L.mapK, L.mapV, L.p);
 }
 
 // The dense variants are always paired (L.p.pair), sparse where two heads

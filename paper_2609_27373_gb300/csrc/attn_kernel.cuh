@@ -565,7 +565,7 @@ struct EpiInfo {
 
 // ------------------------------------------------------------------- softmax
 template <int D, int BLK, int MODE>
-__device__ void attn_softmax(const CUtensorMap* mapO, const AttnParams& p, int w, uint32_t tmem, uint8_t* out_stage,
+__device__ void attn_softmax(const AttnParams& p, int w, uint32_t tmem, uint8_t* out_stage,
                              float* mass_ws,
                              SharedState<AttnCfg<D>::kRingK, AttnCfg<D>::kRingV>& sb) {
   using C = AttnCfg<D>;
@@ -914,10 +914,8 @@ __device__ void attn_softmax(const CUtensorMap* mapO, const AttnParams& p, int w
     j += 2;
   }
   // A warp that gave up inside a tile may still have TMEM stores in flight:
-  // they complete before TMEM is released.  Output stores issued by this
-  // warp complete before the CTA exits.
+  // they complete before TMEM is released.
   tmem_st_wait();
-  if (lane == 0) tma_store_wait_all();
   if (!ok) raise_status(p, &sb.abort, kStatusTimeout);
 }
 
@@ -925,8 +923,7 @@ __device__ void attn_softmax(const CUtensorMap* mapO, const AttnParams& p, int w
 template <int D, int BLK, int MODE>
 __global__ void __launch_bounds__(AttnCfg<D>::kThreads, 1)
     attn_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO,
-                const AttnParams p) {
+                const __grid_constant__ CUtensorMap mapV, const AttnParams p) {
   using C = AttnCfg<D>;
   using SS = SharedState<C::kRingK, C::kRingV>;
   static_assert(sizeof(SS) <= C::kStaticReserve, "static shared memory");
@@ -982,7 +979,6 @@ __global__ void __launch_bounds__(AttnCfg<D>::kThreads, 1)
     tma_prefetch_map(&mapQ);
     tma_prefetch_map(&mapK);
     tma_prefetch_map(&mapV);
-    tma_prefetch_map(&mapO);
   }
   if (warp == C::kMmaSWarp) {
     tmem_alloc(&sb.tmem_base, C::kTmemCols);
@@ -1005,7 +1001,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::kThreads, 1)
 
   if (warp < 8) {
     warpgroup_reg_inc<C::kRegsSoftmax>();
-    attn_softmax<D, BLK, MODE>(&mapO, p, warp >> 2, tmem, out_stage,
+    attn_softmax<D, BLK, MODE>(p, warp >> 2, tmem, out_stage,
                                reinterpret_cast<float*>(out_stage + C::kOutBytes), sb);
   } else {
     warpgroup_reg_dec<C::kRegsOther>();
@@ -1033,24 +1029,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::kThreads, 1)
 template <int D, int BLK, int MODE>
 cudaError_t launch_attn_instance(const AttnLaunch& L) {
   using C = AttnCfg<D>;
-  auto kern = attn_kernel<D, BLK, MODE>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemLaunch);
-  if (e != cudaSuccess) return e;
-  // Programmatic stream serialization: the grid may be scheduled while the
-  // previous kernel of the stream finishes (see griddep_wait in the kernel).
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(L.grid);
-  cfg.blockDim = dim3(C::kThreads);
-  cfg.dynamicSmemBytes = C::kSmemLaunch;
-  cfg.stream = L.stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, L.mapQ, L.mapK, L.mapV, L.mapO, L.p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_dependent<attn_kernel<D, BLK, MODE>>(L.grid, C::kThreads, C::kSmemLaunch, L.stream, L.mapQ, L.mapK, L.mapV, L.p);
 }
 
 template <int D>

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import functools
 import os
 
 import torch
@@ -126,17 +127,35 @@ def status_string(code: int) -> str:
     return load().wise_status_string(int(code)).decode()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+# The small calls are bound by the host (the GPU work of a 512-token late step
+# is 6.6 us): arguments go to ctypes as plain integers, the C structs of a shape
+# and a rule are built once per value, the current stream is read without
+# building a Stream object, and a tensor that is as it should be passes _check
+# with one expression.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
+
+
+def _ptr(t):
+    return None if t is None else t.data_ptr()
+
+
+@functools.lru_cache(maxsize=256)
+def _c(value):
+    """Reference to the C struct of a Shape or Select (read only)."""
+    return ctypes.byref(value.c())
 
 
 def _check(t, name, shape, dtype):
+    if t is not None and t.is_cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous():
+        return
     if t is None:
         raise ValueError(f"{name} is required")
     if not t.is_cuda:
@@ -166,8 +185,7 @@ def wise_full_attn_accumulate(shape: Shape, Q, K, V, O, blockmass=None, step: in
     if blockmass is not None:
         nb = shape.n_blocks
         _check(blockmass, "blockmass", (shape.batch, shape.n_heads, nb, nb), torch.float32)
-    sh = shape.c()
-    rc = load().wise_full_attn_accumulate(ctypes.byref(sh), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(blockmass),
+    rc = load().wise_full_attn_accumulate(_c(shape), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(blockmass),
                                           int(step), _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_full_attn_accumulate")
@@ -182,8 +200,7 @@ def wise_full_attn_accumulate_noalloc(shape: Shape, Q, K, V, O, blockmass, step:
     _qkvo(shape, Q, K, V, O)
     nb = shape.n_blocks
     _check(blockmass, "blockmass", (shape.batch, shape.n_heads, nb, nb), torch.float32)
-    sh = shape.c()
-    rc = load().wise_full_attn_accumulate_noalloc(ctypes.byref(sh), _ptr(Q), _ptr(K), _ptr(V), _ptr(O),
+    rc = load().wise_full_attn_accumulate_noalloc(_c(shape), _ptr(Q), _ptr(K), _ptr(V), _ptr(O),
                                                   _ptr(blockmass), int(step), _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_full_attn_accumulate_noalloc")
@@ -196,8 +213,7 @@ def wise_select_support(shape: Shape, sel: Select, blockmass, idx, counts, strea
     _check(blockmass, "blockmass", (shape.batch, shape.n_heads, nb, nb), torch.float32)
     _check(idx, "idx", (shape.batch, shape.n_kv_heads, nb, sel.cap), torch.int32)
     _check(counts, "counts", (shape.batch, shape.n_kv_heads, nb), torch.int32)
-    sh, se = shape.c(), sel.c()
-    rc = load().wise_select_support(ctypes.byref(sh), ctypes.byref(se), _ptr(blockmass), _ptr(idx), _ptr(counts),
+    rc = load().wise_select_support(_c(shape), _c(sel), _ptr(blockmass), _ptr(idx), _ptr(counts),
                                     _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_select_support")
@@ -212,8 +228,7 @@ def wise_sparse_attn(shape: Shape, Q, K, V, idx, counts, O, stream=None) -> None
     cap = idx.shape[-1]
     _check(idx, "idx", (shape.batch, shape.n_kv_heads, nb, cap), torch.int32)
     _check(counts, "counts", (shape.batch, shape.n_kv_heads, nb), torch.int32)
-    sh = shape.c()
-    rc = load().wise_sparse_attn(ctypes.byref(sh), _ptr(Q), _ptr(K), _ptr(V), _ptr(idx), _ptr(counts), int(cap),
+    rc = load().wise_sparse_attn(_c(shape), _ptr(Q), _ptr(K), _ptr(V), _ptr(idx), _ptr(counts), int(cap),
                                  _ptr(O), _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_sparse_attn")
@@ -229,8 +244,7 @@ def wise_freeze_a_attn(shape: Shape, Q_frozen, K_frozen, V, idx, counts, O, stre
     cap = idx.shape[-1]
     _check(idx, "idx", (shape.batch, shape.n_kv_heads, nb, cap), torch.int32)
     _check(counts, "counts", (shape.batch, shape.n_kv_heads, nb), torch.int32)
-    sh = shape.c()
-    rc = load().wise_freeze_a_attn(ctypes.byref(sh), _ptr(Q_frozen), _ptr(K_frozen), _ptr(V), _ptr(idx),
+    rc = load().wise_freeze_a_attn(_c(shape), _ptr(Q_frozen), _ptr(K_frozen), _ptr(V), _ptr(idx),
                                    _ptr(counts), int(cap), _ptr(O), _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_freeze_a_attn")
@@ -249,8 +263,7 @@ def wise_freeze_a_probs(shape: Shape, Q_frozen, K_frozen, idx, counts, P, inv_l,
     _check(K_frozen, "K_frozen", (shape.batch, shape.n_kv_heads, shape.seqlen, shape.head_dim), torch.bfloat16)
     cap = _support(shape, idx, counts)
     tile_cap = _p_tiles(shape, P, inv_l)
-    sh = shape.c()
-    rc = load().wise_freeze_a_probs(ctypes.byref(sh), _ptr(Q_frozen), _ptr(K_frozen), _ptr(idx), _ptr(counts), cap,
+    rc = load().wise_freeze_a_probs(_c(shape), _ptr(Q_frozen), _ptr(K_frozen), _ptr(idx), _ptr(counts), cap,
                                     _ptr(P), _ptr(inv_l), tile_cap, _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_freeze_a_probs")
@@ -262,8 +275,7 @@ def wise_frozen_pv(shape: Shape, P, inv_l, V, idx, counts, O, stream=None) -> No
     _check(O, "O", (shape.batch, shape.n_heads, shape.seqlen, shape.head_dim), torch.bfloat16)
     cap = _support(shape, idx, counts)
     tile_cap = _p_tiles(shape, P, inv_l)
-    sh = shape.c()
-    rc = load().wise_frozen_pv(ctypes.byref(sh), _ptr(P), _ptr(inv_l), tile_cap, _ptr(V), _ptr(idx), _ptr(counts),
+    rc = load().wise_frozen_pv(_c(shape), _ptr(P), _ptr(inv_l), tile_cap, _ptr(V), _ptr(idx), _ptr(counts),
                                cap, _ptr(O), _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_frozen_pv")
@@ -300,8 +312,7 @@ def wise_support_overlap(shape: Shape, idx_a, counts_a, idx_b, counts_b, inter_u
         _check(idx, name, (shape.batch, shape.n_kv_heads, nb, caps[-1]), torch.int32)
         _check(counts, "counts" + name[3:], (shape.batch, shape.n_kv_heads, nb), torch.int32)
     _check(inter_union, "inter_union", (shape.batch, 2), torch.int64)
-    sh = shape.c()
-    rc = load().wise_support_overlap(ctypes.byref(sh), _ptr(idx_a), _ptr(counts_a), caps[0], _ptr(idx_b),
+    rc = load().wise_support_overlap(_c(shape), _ptr(idx_a), _ptr(counts_a), caps[0], _ptr(idx_b),
                                      _ptr(counts_b), caps[1], _ptr(inter_union), _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_support_overlap")
@@ -320,8 +331,7 @@ def wise_support_mass(shape: Shape, blockmass, idx, counts, retained, stream=Non
     _check(idx, "idx", (shape.batch, shape.n_kv_heads, nb, cap), torch.int32)
     _check(counts, "counts", (shape.batch, shape.n_kv_heads, nb), torch.int32)
     _check(retained, "retained", (shape.batch, shape.n_heads, nb), torch.float32)
-    sh = shape.c()
-    rc = load().wise_support_mass(ctypes.byref(sh), _ptr(blockmass), _ptr(idx), _ptr(counts), cap, _ptr(retained),
+    rc = load().wise_support_mass(_c(shape), _ptr(blockmass), _ptr(idx), _ptr(counts), cap, _ptr(retained),
                                   _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_support_mass")
@@ -352,8 +362,7 @@ def wise_select_working_set(shape: Shape, mode: int, step_masses, idx, counts, e
         ref_cap = int(ref_idx.shape[3])
         _check(ref_idx, "ref_idx", (shape.batch, shape.n_kv_heads, nb, ref_cap), torch.int32)
         _check(ref_counts, "ref_counts", (shape.batch, shape.n_kv_heads, nb), torch.int32)
-    sh = shape.c()
-    rc = load().wise_select_working_set(ctypes.byref(sh), int(mode), float(eta), int(n_sink), int(n_local),
+    rc = load().wise_select_working_set(_c(shape), int(mode), float(eta), int(n_sink), int(n_local),
                                         _ptr(step_masses), n_steps, _ptr(ref_idx), _ptr(ref_counts), ref_cap,
                                         _ptr(idx), _ptr(counts), cap, _stream(stream))
     if rc != WISE_OK:
