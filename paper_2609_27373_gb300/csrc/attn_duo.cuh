@@ -591,7 +591,29 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
   bool due = false, ok = true;
 #pragma unroll 1
   for (;;) {
-    // The next entry, if it is there.
+    // V of the tile whose P V is due.
+    int v_slot = 0;
+    uint32_t v_lo = 0;
+    if (due) {
+      uint64_t* v_bar = &sb.v_full[s];
+      uint32_t v_par = j & 1;
+      const uint8_t* v_at = k_boxes + C::kKBoxes * C::kBox;
+      if constexpr (kPaired) {
+        const int l = 2 * (fl >> 8) + 1;
+        v_slot = l % R;
+        v_bar = &sb.full[v_slot];
+        v_par = (l / R) & 1;
+        v_at = kv + v_slot * C::kTile;
+      }
+      v_lo = low(v_at, C::kBox);
+      if (!duo_warp_wait(v_bar, v_par, abort)) {
+        ok = false;
+        break;
+      }
+    }
+    // The next entry, if it is there (the producer publishes it right after
+    // the copy of that V is started; looked for before the wait above it was
+    // missed at every other tile, and S(j+1) then came 700 clk later).
     const int slot = pos % kDuoSlots;
     const uint32_t slot_par = (pos / kDuoSlots) & 1;
     bool got = __all_sync(0xffffffffu, mbar_test_wait(&sb.sched_full[s][slot], slot_par));
@@ -635,20 +657,8 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
       sb.beat[s] = pos;
     };
     if (due) {
-      int v_slot = 0;
-      uint64_t* v_bar = &sb.v_full[s];
-      uint32_t v_par = j & 1;
-      const uint8_t* v_at = k_boxes + C::kKBoxes * C::kBox;
-      if constexpr (kPaired) {
-        const int l = 2 * (fl >> 8) + 1;
-        v_slot = l % R;
-        v_bar = &sb.full[v_slot];
-        v_par = (l / R) & 1;
-        v_at = kv + v_slot * C::kTile;
-      }
-      const uint32_t b = low(v_at, C::kBox);
       const uint32_t acc = (fl & kEntFirst) ? 0u : 1u;
-      if (!duo_warp_wait(v_bar, v_par, abort) || !duo_warp_wait(&sb.p_full[s], j & 1, abort)) {
+      if (!duo_warp_wait(&sb.p_full[s], j & 1, abort)) {
         ok = false;
         break;
       }
@@ -657,7 +667,7 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         tc_fence_after_sync();
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
-          umma_ts_split(o_tm, s_tm + kk * 8, b + ((kk * 2048) >> 4), v_hi, idesc_o, kk > 0 ? 1u : acc);
+          umma_ts_split(o_tm, s_tm + kk * 8, v_lo + ((kk * 2048) >> 4), v_hi, idesc_o, kk > 0 ? 1u : acc);
         umma_commit(kPaired ? &sb.empty[v_slot] : &sb.v_free[s]);
         if (fl & kEntLast) umma_commit(&sb.o_full[s]);
         chain = next && mbar_test_wait(k_bar, k_par);
