@@ -789,16 +789,23 @@ __device__ __forceinline__ void mask_in_tmem(uint32_t s_col, int diag, int lane)
   tmem_st_wait();
 }
 
-// Blocks of 32 and 64: most tiles have masked keys.
-__device__ __forceinline__ void mask_in_regs(float (&s)[kTileN], uint32_t off, int diag, int lane) {
+// Blocks of 32 and 64, where most tiles have masked keys: the row's maximum
+// over the chunks that are kept, masking the one the diagonal crosses.  Dropped
+// chunks are not touched (their exponentials are skipped as well); set to -inf
+// like the others' masked keys they cost 700 clk a tile.
+__device__ __forceinline__ float masked_row_max(float (&s)[kTileN], uint32_t off, int diag, int lane) {
+  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
   for (int c = 0; c < kTileN / 32; ++c) {
-    const int last = (off >> c) & 1u ? -1 : c == diag ? lane : 31;
-    if (last < 31) {
+    if ((off >> c) & 1u) continue;
+    if (c == diag) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) s[32 * c + i] = i > last ? -INFINITY : s[32 * c + i];
+      for (int i = 1; i < 32; ++i) s[32 * c + i] = i > lane ? -INFINITY : s[32 * c + i];
     }
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) m[(i / 2) & 3] = fmax3(m[(i / 2) & 3], s[32 * c + i], s[32 * c + i + 1]);
   }
+  return fmaxf(fmax3(m[0], m[1], m[2]), m[3]);
 }
 
 // Words w[4 k + q] of a row lie in lane q of a quad (k = 0 .. 4 M - 1 in its
@@ -921,8 +928,7 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
     }
     float s[kTileN];
     tmem_load_row<kTileN>(s_col, s);
-    if (S > 1 && (off != 0u || diag < 4)) mask_in_regs(s, off, diag, lane);
-    const float m_tile = row_max(s) * p.scale_log2;
+    const float m_tile = (S > 1 ? masked_row_max(s, off, diag, lane) : row_max(s)) * p.scale_log2;
     const float m_new = (m_tile > m + kRescaleThreshold) ? m_tile : m;
     const float shift = m_new == -INFINITY ? 0.0f : m_new;
     if (m_new != m) {
@@ -954,7 +960,7 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
       // P of 32 keys, over S, which this warp has read.  Chunks without a key
       // are skipped where there are many (blocks of 32 and 64).
       uint32_t pw[16];
-      if (MODE == kSparse && S > 1 && ((off >> c) & 1u)) {
+      if (S > 1 && ((off >> c) & 1u)) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) pw[e] = 0u;
       } else {
