@@ -769,8 +769,8 @@ __device__ __forceinline__ float sum4(const float2 (&a)[4]) {
 // for the whole warp.
 __device__ __forceinline__ uint32_t masked_key(uint32_t v, int i, int lane) { return i > lane ? 0xFF800000u : v; }
 
-// Block 128: only a unit's last tile has masked keys.  They are set to -inf
-// in tensor memory by a small loop that costs this tile about 700 clk: as
+// Block 128, and the dense variants: only a unit's last tile has masked keys.
+// They are set to -inf in tensor memory by a small loop that costs this tile about 700 clk: as
 // straight-line code on the registers it was fetched from beyond the
 // instruction cache once a unit, 2000 to 4000 clk.
 __device__ __forceinline__ void mask_in_tmem(uint32_t s_col, int diag, int lane) {
@@ -789,7 +789,7 @@ __device__ __forceinline__ void mask_in_tmem(uint32_t s_col, int diag, int lane)
   tmem_st_wait();
 }
 
-// Blocks of 32 and 64, where most tiles have masked keys: the row's maximum
+// Sparse with blocks of 32 and 64, where most tiles have masked keys: the row's maximum
 // over the chunks that are kept, masking the one the diagonal crosses.  Dropped
 // chunks are not touched (their exponentials are skipped as well); set to -inf
 // like the others' masked keys they cost 700 clk a tile.
@@ -917,7 +917,7 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
     int diag = 4;
     if (((uint32_t)ent.x >> 16) != kAllPairs || kt >= qt) {
       diag = (row - lane - kt * kTileN) >> 5;
-      if constexpr (S == 1) {
+      if constexpr (S == 1 || MODE != kSparse) {
         mask_in_tmem(s_col, diag, lane);
       } else {
         const uint32_t sub = (uint32_t)ent.x >> (16 + qsub * S);
@@ -928,7 +928,8 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
     }
     float s[kTileN];
     tmem_load_row<kTileN>(s_col, s);
-    const float m_tile = (S > 1 ? masked_row_max(s, off, diag, lane) : row_max(s)) * p.scale_log2;
+    constexpr bool kChunks = MODE == kSparse && S > 1;  // chunks of 32 keys one by one
+    const float m_tile = (kChunks ? masked_row_max(s, off, diag, lane) : row_max(s)) * p.scale_log2;
     const float m_new = (m_tile > m + kRescaleThreshold) ? m_tile : m;
     const float shift = m_new == -INFINITY ? 0.0f : m_new;
     if (m_new != m) {
@@ -960,7 +961,7 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
       // P of 32 keys, over S, which this warp has read.  Chunks without a key
       // are skipped where there are many (blocks of 32 and 64).
       uint32_t pw[16];
-      if (S > 1 && ((off >> c) & 1u)) {
+      if (kChunks && ((off >> c) & 1u)) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) pw[e] = 0u;
       } else {

@@ -136,21 +136,20 @@ bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long
 // Whether a launch runs on attn_duo_kernel (two query tiles in flight per CTA)
 // rather than attn_kernel (both softmax warpgroups on one), and its pairing.
 // With few units a CTA of the former has no second one to overlap with the
-// first, and a unit alone takes longer there.  Measured (us, attn_kernel /
-// attn_duo_kernel; d = head dim):
-//   dense: 256 units (2K, 16 heads, d 128) 20.2 / 28.9, 384 (4K, 12 heads) 47.5 / 52.0,
-//     512 (4K, 16 heads) 57.3 / 52.8, 1024 (4K, 32 heads) 119 / 105;
-//   sparse, block 128, d 128: 384 27.6 / 29.9, 512 (4K) 32.7 / 33.4, 512 (8K) 42.0 /
-//     40.4, 1024 (8K) 74.3 / 71.1, 1024 (4K, 32 heads) 63 / 58; d 96: 768 44.2 / 43.0;
-//   sparse, block 32 or 64, or d 64: 192 19.9 / 26.6, 512 (d 64, block 64) 37.2 / 29.0,
-//     512 (d 128, block 64) 62.7 / 55.6, 512 (d 64, block 64, 512 tokens) 19.7 / 15.3.
+// first, and a unit alone takes longer there.  Measured back to back in a graph
+// (us, attn_kernel / attn_duo_kernel; d = head dim, B = block):
+//   dense: 256 units (2K, 16 heads, d 128) 19.3 / 28.2, 384 (4K, 12 heads) 45.9 / 51.1,
+//     512 (4K, 16 heads) 55.9 / 51.7, 640 (4K, 20 heads) 70.2 / 64.2;
+//   sparse, B 128, d 128: 384 (4K) 26.6 / 28.2, 512 (4K) 31.9 / 32.0, 512 (8K) 41.0 /
+//     37.9, 640 (4K) 38.8 / 35.4; d 96: 768 43.7 / 40.2;
+//   sparse, smaller blocks: 192 (4K, d 128, B 64) 29.9 / 35.6, 512 (4K, d 128, B 64)
+//     61.9 / 52.4, 512 (2K, d 64, B 64) 36.5 / 29.2.
 // The line depends on the shape alone, not on the variant: sparse attention
 // over every block and dense attention run on the same kernel and give the
 // same bits.
-bool choose_duo(int mode, const wise_shape_t* sh, int sm_count, AttnParams& p) {
+bool choose_duo(int mode, int sm_count, AttnParams& p) {
   if (p.n_qtiles > 256) return false;  // the staged tile masks hold 256 key tiles
-  const bool wide = sh->block == 128 && sh->head_dim > 64;
-  if (p.n_units < (wide ? 4 : 3) * sm_count) return false;
+  if (p.n_units < 3 * sm_count) return false;
   p.pair = kPairNone;
   p.v_heads = p.n_heads;
   p.v_qtiles = p.n_qtiles;
@@ -251,7 +250,7 @@ int launch_attention(const wise_shape_t* sh, const void* Q, const void* K, const
     }
   }
   cudaError_t e;
-  if (choose_duo(mode, sh, ds->sm_count, p)) {
+  if (choose_duo(mode, ds->sm_count, p)) {
     p.o_align32 = aligned(O, 32);
     L.grid = std::min(p.v_units, ds->sm_count);
     switch (sh->head_dim) {
