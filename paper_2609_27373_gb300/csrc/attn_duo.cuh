@@ -49,7 +49,7 @@
 // 440, exponentials and P 730 (550 of it the ex2 rate, 4.3 clk per warp
 // instruction), 450 until P V is issued, S(j+1) 440 behind it.  attn_kernel
 // takes 1930 clk a tile.  Measured against it (us, attn_kernel / here): dense
-// 119 / 105, dense + mass 128 / 115, sparse block 128 64 / 58, block 32 150 / 120;
+// 119 / 105, dense + mass 128 / 112, sparse block 128 64 / 58, block 32 150 / 120;
 // 16K sparse 355 / 300; 32K, four heads to a kv head 850 / 705 (paired); 4 x 4K,
 // head dim 96 405 / 330.
 //
@@ -132,7 +132,6 @@ struct DuoShared {
   uint32_t tmem_base;
   int abort;
   int beat[2];  // tiles begun by each stream
-  int issuing;  // the streams' turn at issuing products (0 free, 1 taken)
 };
 
 // Unit u -> (batch, virtual head, virtual query tile): see decode_unit; a
@@ -565,24 +564,6 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
   const uint32_t s_tm = tmem + C::kTmemS + s * 128, o_tm = tmem + C::kTmemO + s * 128;
   const uint8_t* k_boxes = kv + s * C::kStream;  // unpaired
 
-  // The streams of a paired launch take turns at issuing, a P V with the S
-  // behind it at a time.  With their products interleaved both streams' would
-  // end together, and both softmaxes then run at once while the tensor pipe
-  // idles (4K dense 113 us without turns, 108 with); unpaired streams, whose
-  // loads keep them apart, only lose time by it (4K sparse 58 and 64 us).
-  // Leader only; false when the launch was aborted meanwhile.
-  auto lock = [&]() -> bool {
-    if constexpr (kPaired) {
-#pragma unroll 1
-      while (atomicCAS(&sb.issuing, 0, 1) != 0)
-        if (*abort) return false;
-    }
-    return true;
-  };
-  auto unlock = [&]() {
-    if constexpr (kPaired) atomicExch(&sb.issuing, 0);
-  };
-
   int pos = 0;  // entries taken
   int j = 0;    // tiles whose P V has been issued
   int nq = 0;   // units begun
@@ -648,7 +629,6 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         umma_ss_split(s_tm, q_lo + (kk >> 2) * (C::kBox >> 4) + off, k_hi, (kk < 4 ? k0 : k1) + off, k_hi, idesc_s,
                       kk > 0 ? 1u : 0u);
       }
-      unlock();
       umma_commit(&sb.s_full[s]);
       if constexpr (kPaired) {
         umma_commit(&sb.empty[k_slot]);
@@ -663,7 +643,6 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         break;
       }
       if (leader) {
-        ok = lock();
         tc_fence_after_sync();
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
@@ -671,17 +650,11 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         umma_commit(kPaired ? &sb.empty[v_slot] : &sb.v_free[s]);
         if (fl & kEntLast) umma_commit(&sb.o_full[s]);
         chain = next && mbar_test_wait(k_bar, k_par);
-        if (chain) {
-          issue_s();
-        } else {
-          unlock();
-        }
+        if (chain) issue_s();
         if (kPaired && (fl & kEntSolo)) umma_commit(&sb.empty[v_slot]);
         mbar_arrive(&sb.sched_empty[s][(pos - 1) % kDuoSlots]);
       }
       chain = __any_sync(0xffffffffu, chain);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
       due = false;
       ++j;
     }
@@ -719,12 +692,10 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         break;
       }
       if (leader) {
-        ok = lock();
         tc_fence_after_sync();
         issue_s();
       }
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
+      __syncwarp();
     }
     fl = ent.z;
     due = true;
@@ -1089,7 +1060,6 @@ __global__ void __launch_bounds__(512, 1)
   }
   if (threadIdx.x == 0) {
     sb.abort = 0;
-    sb.issuing = 0;
     sb.beat[0] = sb.beat[1] = 0;
     sb.stage.next = 0;
     for (int i = 0; i < C::kRing; ++i) {
