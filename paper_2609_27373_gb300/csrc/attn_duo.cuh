@@ -30,9 +30,9 @@
 //
 // Shared memory at head dim 128: a Q tile per stream (2 x 32 KB) and five
 // more tiles.  Paired, they are one ring of K and V tiles.  Unpaired, each
-// stream has one V tile and one and a half K tiles (three 64-column boxes):
-// with rings of their own a stream that stands still does not hold up the
-// other's loads.  That leaves 3 KB for everything else (hence the packed tile
+// stream has one V tile and one and a half K tiles (three 64-column boxes; at
+// head dim 96 two V tiles and five 32-column boxes): with rings of their own a
+// stream that stands still does not hold up the other's loads.  That leaves 3 KB for everything else (hence the packed tile
 // masks and the small schedule rings).
 //
 // Warp roles (512 threads; warps 14 and 15 only complete the warpgroup):
@@ -71,7 +71,11 @@ constexpr int kEntSolo = 64;        // the tile is used by this stream only (pai
 // Units staged by warp 12.
 template <int S, bool kMask>
 struct DuoStage {
-  static constexpr int kSlots = 2;  // units staged ahead
+  // Units staged ahead.  At least two: a producer that takes the unit of a
+  // slot then knows the slot's earlier phase complete (the unit two before has
+  // been taken); with one, the second producer may wait for a phase while the
+  // one before it is still open, and a parity wait would return at once.
+  static constexpr int kSlots = 2;
   // Sparse: S * S bits per key tile, packed.
   static constexpr int kWords = kMask ? kDuoStageTiles * S * S / 32 : 1;
   uint64_t full[kSlots], empty[kSlots];
@@ -88,17 +92,25 @@ struct DuoNoMass {};
 
 template <int D, bool kPaired>
 struct DuoCfg {
-  static constexpr int kBoxes = (D + 63) / 64;
-  static constexpr int kBox = 128 * 128;            // bytes of a 128-row, 64-column box
+  // 128-row boxes of 64 columns (128-byte swizzle).  Unpaired at head dim 96,
+  // of 32 columns (64-byte swizzle): a tile then takes 24 KB instead of 32
+  // (half of the second 64-column box is not used), and a stream has room for a
+  // second V tile (4 x 4K, 55 heads: 316 -> 305 us; block 32, 2 x 4K, 32 heads:
+  // 204 -> 200).  Paired launches gained nothing from 7 ring entries instead of
+  // 5, and dense + mass lost 1 %.
+  static constexpr int kCols = duo_box_cols(D, kPaired);
+  static constexpr int kBoxes = (D + kCols - 1) / kCols;
+  static constexpr int kBox = 128 * kCols * 2;      // bytes
   static constexpr int kTile = kBoxes * kBox;       // bytes of a 128-row Q, K or V tile
   static constexpr int kBudget = 227 * 1024;
   static constexpr int kStateBytes = (D > 64 ? 3 : 4) * 1024;
   // Paired: ring of K and V tiles.
   static constexpr int kFit = (kBudget - kStateBytes - 2 * kTile) / kTile;
   static constexpr int kRing = kFit > 8 ? 8 : kFit;
-  // Unpaired, per stream: K boxes (used as a ring) and one V tile.
-  static constexpr int kKBoxes = kBoxes + 1;
-  static constexpr int kStream = kKBoxes * kBox + kTile;
+  // Unpaired, per stream: K boxes (used as a ring) and one or two V tiles.
+  static constexpr int kVTiles = kCols == 32 ? 2 : 1;
+  static constexpr int kKBoxes = 2 * kBoxes - (D == 64 ? 0 : 1);
+  static constexpr int kStream = kKBoxes * kBox + kVTiles * kTile;
   static constexpr int kKVBytes = kPaired ? kRing * kTile : 2 * kStream;
   // The dynamic shared memory of a kernel without static shared memory starts
   // 1024-byte aligned (checked by the kernel's set-up).  At least 116 KB, so
@@ -117,7 +129,7 @@ struct DuoShared {
   static constexpr int S = kTileN / BLK;
   using Stage = DuoStage<S, MODE == kSparse>;
   uint64_t full[R], empty[R];                // paired: K/V ring
-  uint64_t k_full[2][2], v_full[2], v_free[2];  // unpaired: K(j) by j & 1; V(j) landed; P V(j) complete
+  uint64_t k_full[2][2], v_full[2][2], v_free[2];  // unpaired: K(j), V(j) landed, by j & 1; P V(j) complete
   uint64_t sched_full[2][kDuoSlots], sched_empty[2][kDuoSlots];  // schedule entry written / read by all
   uint64_t q_full[2];
   uint64_t s_full[2];     // S(j) complete, and with it P V(j-1)
@@ -379,10 +391,12 @@ __device__ __forceinline__ bool duo_emit(const AttnParams& p, int s, int& pos, i
   return true;
 }
 
-// Unpaired: stream s's producer (lane 0 does the loads).  K(j) goes to the
-// boxes 2 j and 2 j + 1 of the K ring (modulo 3; at head dim 64 box j modulo
-// 2).  Box 0 is free once S(j-2) has completed, which V(j-1)'s wait implies,
-// box 1 once S(j-1) has, and the V tile once P V(j-1) has.
+// Unpaired: stream s's producer (lane 0 does the loads).  The boxes of K(j)
+// follow those of K(j-1) in a ring of one box less than two tiles (two tiles at
+// head dim 64): all but the last are free once S(j-2) has completed, which
+// V(j-1)'s wait or the one for the last box of K(j-1) has seen, the last one
+// once S(j-1) has.  With one V tile, V(j) may be loaded once P V(j-1) is
+// complete; with two, once P V(j-2) is, and S(j-1) complete means that.
 template <int D, int BLK, int MODE, class Sh>
 __device__ void duo_producer(const CUtensorMap* mapK, const CUtensorMap* mapV, const AttnParams& p, int s,
                              uint8_t* kv, Sh& sb) {
@@ -390,7 +404,7 @@ __device__ void duo_producer(const CUtensorMap* mapK, const CUtensorMap* mapV, c
   const int lane = threadIdx.x & 31;
   volatile int* abort = &sb.abort;
   uint8_t* k_boxes = kv + s * C::kStream;
-  uint8_t* v_tile = k_boxes + C::kKBoxes * C::kBox;
+  uint8_t* v_tiles = k_boxes + C::kKBoxes * C::kBox;
   int pos = 0, j = 0, box = 0, nk = 0, nv = 0;  // tiles, next K box, K and V tiles loaded
   bool ok = true, waited = false;
   for (;;) {
@@ -419,25 +433,26 @@ __device__ void duo_producer(const CUtensorMap* mapK, const CUtensorMap* mapV, c
         }
         uint64_t* k_full = &sb.k_full[s][j & 1];
         mbar_arrive_expect_tx(k_full, C::kTile);
-        tma_load_3d(k_boxes + box * C::kBox, mapK, k_full, 0, y, unit.z);
-        box = box + 1 == C::kKBoxes ? 0 : box + 1;
-        if constexpr (C::kBoxes == 2) {
-          const bool free = j < 1 || duo_wait(&sb.s_full[s], (j - 1) & 1, abort);
-          // Issued in any case: the barrier expects the whole tile.  (After a
-          // wait that gave up nothing is read from it any more.)
-          tma_load_3d(k_boxes + box * C::kBox, mapK, k_full, 64, y, unit.z);
+        bool free = true;
+#pragma unroll
+        for (int i = 0; i < C::kBoxes; ++i) {
+          // Issued after a wait that gave up as well: the barrier expects the
+          // whole tile, and nothing is read from it any more.
+          if (D > 64 && i + 1 == C::kBoxes) free = j < 1 || duo_wait(&sb.s_full[s], (j - 1) & 1, abort);
+          tma_load_3d(k_boxes + box * C::kBox, mapK, k_full, C::kCols * i, y, unit.z);
           box = box + 1 == C::kKBoxes ? 0 : box + 1;
-          if (!free) ok = false;
         }
         ++nk;
-        if (!ok || (j >= 1 && !duo_wait(&sb.v_free[s], (j - 1) & 1, abort))) {
+        if (C::kVTiles == 1 && free) free = j < 1 || duo_wait(&sb.v_free[s], (j - 1) & 1, abort);
+        if (!free) {
           ok = false;
           break;
         }
-        mbar_arrive_expect_tx(&sb.v_full[s], C::kTile);
+        const int v_buf = C::kVTiles == 1 ? 0 : j & 1;
+        mbar_arrive_expect_tx(&sb.v_full[s][v_buf], C::kTile);
 #pragma unroll
         for (int i = 0; i < C::kBoxes; ++i)
-          tma_load_3d(v_tile + i * C::kBox, mapV, &sb.v_full[s], 64 * i, y, unit.z);
+          tma_load_3d(v_tiles + v_buf * C::kTile + i * C::kBox, mapV, &sb.v_full[s][v_buf], C::kCols * i, y, unit.z);
         ++nv;
       }
     }
@@ -448,7 +463,8 @@ __device__ void duo_producer(const CUtensorMap* mapK, const CUtensorMap* mapV, c
     raise_status(p, &sb.abort, kStatusTimeout);
     // Copies already issued land before shared memory is released.
     for (int i = max(0, nk - 2); i < nk; ++i) duo_drain(&sb.k_full[s][i & 1], (i >> 1) & 1);
-    if (nv > 0) duo_drain(&sb.v_full[s], (nv - 1) & 1);
+    for (int i = max(0, nv - C::kVTiles); i < nv; ++i)
+      duo_drain(&sb.v_full[s][i % C::kVTiles], (i / C::kVTiles) & 1);
   }
 }
 
@@ -477,7 +493,7 @@ __device__ void duo_producer_paired(const CUtensorMap* mapK, const CUtensorMap* 
     mbar_arrive_expect_tx(&sb.full[slot], C::kTile);
 #pragma unroll
     for (int i = 0; i < C::kBoxes; ++i)
-      tma_load_3d(ring + slot * C::kTile + i * C::kBox, map, &sb.full[slot], 64 * i, y, z);
+      tma_load_3d(ring + slot * C::kTile + i * C::kBox, map, &sb.full[slot], C::kCols * i, y, z);
     step();
   };
   int loads = 0;
@@ -548,6 +564,8 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
                         uint8_t* kv, Sh& sb) {
   using C = DuoCfg<D, kPaired>;
   constexpr int R = C::kRing;
+  constexpr int kRow = C::kCols * 2;   // bytes of a box row, and its swizzle
+  constexpr int kSteps = C::kCols / 16;  // products (of 16 columns) per box
   constexpr uint32_t idesc_s = idesc_bf16_f32(128, kTileN, false, false);
   constexpr uint32_t idesc_o = idesc_bf16_f32(128, D, false, true);
   volatile int* abort = &sb.abort;
@@ -555,10 +573,9 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
   // Shared-memory descriptors: constant high halves, low halves that hold the
   // address.
   auto low = [](const uint8_t* at, uint32_t lbo) {
-    return __shfl_sync(0xffffffffu, (uint32_t)smem_desc_sw128(smem_u32(at), lbo, 1024), 0);
+    return __shfl_sync(0xffffffffu, (uint32_t)smem_desc<kRow>(smem_u32(at), lbo, 8 * kRow), 0);
   };
-  const uint32_t k_hi = (uint32_t)(smem_desc_sw128(0, 16, 1024) >> 32);
-  const uint32_t v_hi = (uint32_t)(smem_desc_sw128(0, C::kBox, 1024) >> 32);
+  constexpr uint32_t hi = (uint32_t)(smem_desc<kRow>(0, 0, 8 * kRow) >> 32);
   uint8_t* q_tile = q_tiles + s * C::kTile;
   const uint32_t q_lo = low(q_tile, 16);
   const uint32_t s_tm = tmem + C::kTmemS + s * 128, o_tm = tmem + C::kTmemO + s * 128;
@@ -576,9 +593,10 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
     int v_slot = 0;
     uint32_t v_lo = 0;
     if (due) {
-      uint64_t* v_bar = &sb.v_full[s];
-      uint32_t v_par = j & 1;
-      const uint8_t* v_at = k_boxes + C::kKBoxes * C::kBox;
+      const int v_buf = C::kVTiles == 1 ? 0 : j & 1;
+      uint64_t* v_bar = &sb.v_full[s][v_buf];
+      uint32_t v_par = (C::kVTiles == 1 ? j : j >> 1) & 1;
+      const uint8_t* v_at = k_boxes + C::kKBoxes * C::kBox + v_buf * C::kTile;
       if constexpr (kPaired) {
         const int l = 2 * (fl >> 8) + 1;
         v_slot = l % R;
@@ -601,7 +619,7 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
     int4 ent = make_int4(0, 0, 0, 0);
     int k_slot = 0;
     uint64_t* k_bar = nullptr;
-    uint32_t k_par = 0, k0 = 0, k1 = 0;  // K: barrier, descriptors of its boxes
+    uint32_t k_par = 0, k_lo[C::kBoxes] = {};  // K: barrier, descriptors of its boxes
     auto look = [&](int jn) {            // jn: the tile of the entry
       ent = sb.sched[s][slot];
       if constexpr (kPaired) {
@@ -609,13 +627,16 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         k_slot = l % R;
         k_bar = &sb.full[k_slot];
         k_par = (l / R) & 1;
-        k0 = low(kv + k_slot * C::kTile, 16);
-        k1 = k0 + (C::kBox >> 4);
+        const uint32_t k0 = low(kv + k_slot * C::kTile, 16);
+#pragma unroll
+        for (int i = 0; i < C::kBoxes; ++i) k_lo[i] = k0 + i * (C::kBox >> 4);
       } else {
         k_bar = &sb.k_full[s][jn & 1];
         k_par = (jn >> 1) & 1;
-        k0 = low(k_boxes + box * C::kBox, 16);
-        k1 = low(k_boxes + (box + 1 == C::kKBoxes ? 0 : box + 1) * C::kBox, 16);
+        const uint32_t k0 = low(k_boxes, 16);
+#pragma unroll
+        for (int i = 0; i < C::kBoxes; ++i)
+          k_lo[i] = k0 + (box + i - (box + i >= C::kKBoxes ? C::kKBoxes : 0)) * (C::kBox >> 4);
       }
     };
     if (got) look(j + (due ? 1 : 0));
@@ -625,9 +646,9 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
     auto issue_s = [&]() {
 #pragma unroll
       for (int kk = 0; kk < D / 16; ++kk) {
-        const uint32_t off = ((kk & 3) * 32) >> 4;
-        umma_ss_split(s_tm, q_lo + (kk >> 2) * (C::kBox >> 4) + off, k_hi, (kk < 4 ? k0 : k1) + off, k_hi, idesc_s,
-                      kk > 0 ? 1u : 0u);
+        const int i = kk / kSteps;
+        const uint32_t off = ((kk % kSteps) * 32) >> 4;
+        umma_ss_split(s_tm, q_lo + i * (C::kBox >> 4) + off, hi, k_lo[i] + off, hi, idesc_s, kk > 0 ? 1u : 0u);
       }
       umma_commit(&sb.s_full[s]);
       if constexpr (kPaired) {
@@ -646,8 +667,8 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         tc_fence_after_sync();
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
-          umma_ts_split(o_tm, s_tm + kk * 8, v_lo + ((kk * 2048) >> 4), v_hi, idesc_o, kk > 0 ? 1u : acc);
-        umma_commit(kPaired ? &sb.empty[v_slot] : &sb.v_free[s]);
+          umma_ts_split(o_tm, s_tm + kk * 8, v_lo + ((kk * 16 * kRow) >> 4), hi, idesc_o, kk > 0 ? 1u : acc);
+        if (kPaired || C::kVTiles == 1) umma_commit(kPaired ? &sb.empty[v_slot] : &sb.v_free[s]);
         if (fl & kEntLast) umma_commit(&sb.o_full[s]);
         chain = next && mbar_test_wait(k_bar, k_par);
         if (chain) issue_s();
@@ -678,7 +699,7 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
           mbar_arrive_expect_tx(&sb.q_full[s], C::kTile);
 #pragma unroll 1
           for (int i = 0; i < C::kBoxes; ++i)
-            tma_load_3d(q_tile + i * C::kBox, mapQ, &sb.q_full[s], 64 * i, (ent.w >> 16) * 128, ent.y);
+            tma_load_3d(q_tile + i * C::kBox, mapQ, &sb.q_full[s], C::kCols * i, (ent.w >> 16) * 128, ent.y);
         }
         __syncwarp();
         ++nq;
@@ -1018,13 +1039,13 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
     // first pass from beyond the instruction cache): rows lane / 4 and
     // lane / 4 + 8 of them in each lane.
 #pragma unroll 1
-    for (int i = 0; i < 2 * C::kBoxes; ++i) {
+    for (int i = 0; i < 2 * ((D + 63) / 64); ++i) {
       const int h = i & 1, c0 = (i >> 1) * 64;
       const int ra = 16 * h + (lane >> 2), rb = ra + 8;
       const float fa = __shfl_sync(0xffffffffu, inv_l, ra), fb = __shfl_sync(0xffffffffu, inv_l, rb);
       const int row0 = qt * 128 + wq * 32;
       __nv_bfloat16* da = p.O + ((size_t)ent.y * p.seqlen + row0 + ra) * D + c0;
-      // At head dim 96 the second box holds 32 columns: the TMEM columns after
+      // At head dim 96 the second pass has 32 columns: the TMEM columns after
       // them are read but not stored.
       uint32_t v[32];
       tmem_ld_16x256b_x8(o_col + ((uint32_t)(16 * h) << 16) + c0, v);
@@ -1073,7 +1094,8 @@ __global__ void __launch_bounds__(512, 1)
       }
       mbar_init(&sb.k_full[s][0], 1);
       mbar_init(&sb.k_full[s][1], 1);
-      mbar_init(&sb.v_full[s], 1);
+      mbar_init(&sb.v_full[s][0], 1);
+      mbar_init(&sb.v_full[s][1], 1);
       mbar_init(&sb.v_free[s], 1);
       mbar_init(&sb.q_full[s], 1);
       mbar_init(&sb.s_full[s], 1);

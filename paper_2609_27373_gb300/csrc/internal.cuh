@@ -52,6 +52,9 @@ struct AttnParams {
   int o_align32;  // O is 32-byte aligned
 };
 
+// Columns of a Q, K or V box of attn_duo_kernel (DuoCfg::kCols).
+constexpr int duo_box_cols(int d, bool paired) { return d == 96 && !paired ? 32 : 64; }
+
 struct AttnLaunch {
   CUtensorMap mapQ, mapK, mapV;
   AttnParams p;

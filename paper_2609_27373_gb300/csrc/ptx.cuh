@@ -186,15 +186,22 @@ __device__ __forceinline__ void tc_fence_after_sync() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle.  lbo/sbo in bytes.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+// Shared-memory matrix descriptor, swizzled in spans of kSwizzle (128 or 64)
+// bytes.  lbo/sbo in bytes.
+template <int kSwizzle>
+__host__ __device__ constexpr uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  static_assert(kSwizzle == 128 || kSwizzle == 64, "swizzle");
   uint64_t d = 0;
   d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
   d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
   d |= static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32;
   d |= static_cast<uint64_t>(1) << 46;  // descriptor version for sm_100-class parts
-  d |= static_cast<uint64_t>(2) << 61;  // 128-byte swizzle
+  d |= static_cast<uint64_t>(kSwizzle == 128 ? 2 : 4) << 61;  // swizzle mode
   return d;
+}
+
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return smem_desc<128>(saddr, lbo, sbo);
 }
 
 // Instruction descriptor of tcgen05.mma kind::f16: bf16 A and B, fp32

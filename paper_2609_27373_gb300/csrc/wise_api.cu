@@ -119,17 +119,20 @@ int check_shape(const wise_shape_t* sh, bool attention) {
   return WISE_OK;
 }
 
-// Tensor map over a [rows_outer, seqlen, head_dim] bf16 array with 64-column,
-// box_rows-row boxes in the 128-byte swizzle.  Rows past seqlen read as zero.
-bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long long outer, int box_rows) {
+// Tensor map over a [rows_outer, seqlen, head_dim] bf16 array with box_rows-row
+// boxes of 64 columns in the 128-byte swizzle or of 32 columns in the 64-byte
+// one.  Rows past seqlen read as zero.
+bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long long outer, int box_rows,
+              int box_cols = 64) {
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)seqlen, (cuuint64_t)outer};
   cuuint64_t strides[2] = {(cuuint64_t)head_dim * 2, (cuuint64_t)head_dim * 2 * (cuuint64_t)seqlen};
-  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1};
   cuuint32_t elem[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -192,11 +195,6 @@ int launch_attention(const wise_shape_t* sh, const void* Q, const void* K, const
   AttnLaunch L;
   const long long outer_q = (long long)sh->batch * sh->n_heads;
   const long long outer_kv = (long long)sh->batch * sh->n_kv_heads;
-  if (!make_map(&L.mapQ, Q, sh->head_dim, sh->seqlen, outer_q, 128) ||
-      !make_map(&L.mapK, K, sh->head_dim, sh->seqlen, outer_kv, 128) ||
-      !make_map(&L.mapV, V, sh->head_dim, sh->seqlen, outer_kv, 128))
-    return WISE_ERR_CUDA;
-
   AttnParams& p = L.p;
   p.batch = sh->batch;
   p.seqlen = sh->seqlen;
@@ -249,8 +247,14 @@ int launch_attention(const wise_shape_t* sh, const void* Q, const void* K, const
       if (!p.scratch) return WISE_ERR_CUDA;
     }
   }
+  const bool duo = choose_duo(mode, ds->sm_count, p);
+  const int cols = duo ? duo_box_cols(sh->head_dim, p.pair != kPairNone) : 64;
+  if (!make_map(&L.mapQ, Q, sh->head_dim, sh->seqlen, outer_q, 128, cols) ||
+      !make_map(&L.mapK, K, sh->head_dim, sh->seqlen, outer_kv, 128, cols) ||
+      !make_map(&L.mapV, V, sh->head_dim, sh->seqlen, outer_kv, 128, cols))
+    return WISE_ERR_CUDA;
   cudaError_t e;
-  if (choose_duo(mode, ds->sm_count, p)) {
+  if (duo) {
     p.o_align32 = aligned(O, 32);
     L.grid = std::min(p.v_units, ds->sm_count);
     switch (sh->head_dim) {

@@ -16,11 +16,12 @@ pytestmark = pytest.mark.gpu
 
 # batch, heads, kv heads, seqlen, head dim, block: unpaired heads with an odd
 # and an even number of query tiles, odd and even groups (head pairs), ragged
-# last tiles at block 32 and 64, one-tile units, more units than a CTA stages.
+# last tiles at block 32 and 64, one-tile units, more units than a CTA stages,
+# unpaired heads of 96 (boxes of their own) over several tiles.
 SHAPES = [
     (4, 52, 52, 384, 128, 128), (2, 40, 40, 1024, 128, 128), (4, 33, 11, 640, 128, 128), (4, 64, 16, 384, 128, 128),
     (4, 55, 55, 384, 96, 128), (3, 54, 9, 544, 96, 32), (4, 40, 40, 576, 64, 64), (4, 64, 32, 416, 64, 32),
-    (8, 80, 80, 128, 64, 128), (10, 64, 8, 96, 64, 32),
+    (8, 80, 80, 128, 64, 128), (10, 64, 8, 96, 64, 32), (2, 37, 37, 1120, 96, 32),
 ]
 
 
