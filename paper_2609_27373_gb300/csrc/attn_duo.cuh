@@ -826,11 +826,22 @@ __device__ __forceinline__ void quad_rows(const uint32_t (&w)[4 * M], int lane, 
   }
 }
 
+// 16 columns of O.
+__device__ __forceinline__ void store_16(__nv_bfloat16* dst, const uint32_t (&q)[8], bool wide) {
+  if (wide) {
+    st_global_v8(dst, q);
+  } else {
+    *reinterpret_cast<uint4*>(dst) = make_uint4(q[0], q[1], q[2], q[3]);
+    *reinterpret_cast<uint4*>(dst + 8) = make_uint4(q[4], q[5], q[6], q[7]);
+  }
+}
+
 // Writes the first `cols` of 64 columns of 8 rows from a fragment
 // (`acc[4 k + at]` and the next: columns 8 k + 2 (lane % 4) of row lane / 4),
 // scaled by the row's f: each lane ends with 16 consecutive columns, so that a
 // warp's store covers whole 128-byte row segments of 8 rows.  (Each thread
-// storing the row it owns took 2300 clk a unit: 32 lines per store.)
+// storing the row it owns took 2300 clk a unit with 16-byte stores: 32 lines
+// per store.)
 __device__ __forceinline__ void store_fragment(__nv_bfloat16* dst, const uint32_t (&acc)[32], int at, float f, int lane,
                                                int cols, bool in, bool wide) {
   uint32_t w[8], q[8];
@@ -843,13 +854,7 @@ __device__ __forceinline__ void store_fragment(__nv_bfloat16* dst, const uint32_
   }
   quad_rows<2>(w, lane, q);
   const int c = 16 * (lane & 3);
-  if (!in || c >= cols) return;
-  if (wide) {
-    st_global_v8(dst + c, q);
-  } else {
-    *reinterpret_cast<uint4*>(dst + c) = make_uint4(q[0], q[1], q[2], q[3]);
-    *reinterpret_cast<uint4*>(dst + c + 8) = make_uint4(q[4], q[5], q[6], q[7]);
-  }
+  if (in && c < cols) store_16(dst + c, q, wide);
 }
 
 template <int D, int BLK, int MODE, class Sh>
@@ -1035,24 +1040,54 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
     tc_fence_after_sync();
     const float inv_l = l > 0.0f ? 1.0f / l : 0.0f;
     const bool wide = p.o_align32 != 0;
-    // Rolled, 16 rows x 64 columns at a time (this code runs once a unit, its
-    // first pass from beyond the instruction cache): rows lane / 4 and
-    // lane / 4 + 8 of them in each lane.
+    if constexpr (D % 64 == 0 || MODE == kDense) {
+      // Rolled, 16 rows x 64 columns at a time (this code runs once a unit, its
+      // first pass from beyond the instruction cache): rows lane / 4 and
+      // lane / 4 + 8 of them in each lane.  At head dim 96 the second 64 have
+      // 32 columns: the TMEM columns after them are read but not stored.
 #pragma unroll 1
-    for (int i = 0; i < 2 * ((D + 63) / 64); ++i) {
-      const int h = i & 1, c0 = (i >> 1) * 64;
-      const int ra = 16 * h + (lane >> 2), rb = ra + 8;
-      const float fa = __shfl_sync(0xffffffffu, inv_l, ra), fb = __shfl_sync(0xffffffffu, inv_l, rb);
-      const int row0 = qt * 128 + wq * 32;
-      __nv_bfloat16* da = p.O + ((size_t)ent.y * p.seqlen + row0 + ra) * D + c0;
-      // At head dim 96 the second pass has 32 columns: the TMEM columns after
-      // them are read but not stored.
-      uint32_t v[32];
-      tmem_ld_16x256b_x8(o_col + ((uint32_t)(16 * h) << 16) + c0, v);
-      tmem_ld_wait(v);
-      const int q_cols = D % 64 == 0 ? 64 : min(D - c0, 64);
-      store_fragment(da, v, 0, fa, lane, q_cols, row0 + ra < p.seqlen, wide);
-      store_fragment(da + 8 * D, v, 2, fb, lane, q_cols, row0 + rb < p.seqlen, wide);
+      for (int i = 0; i < 2 * ((D + 63) / 64); ++i) {
+        const int h = i & 1, c0 = (i >> 1) * 64;
+        const int ra = 16 * h + (lane >> 2), rb = ra + 8;
+        const float fa = __shfl_sync(0xffffffffu, inv_l, ra), fb = __shfl_sync(0xffffffffu, inv_l, rb);
+        const int row0 = qt * 128 + wq * 32;
+        __nv_bfloat16* da = p.O + ((size_t)ent.y * p.seqlen + row0 + ra) * D + c0;
+        uint32_t v[32];
+        tmem_ld_16x256b_x8(o_col + ((uint32_t)(16 * h) << 16) + c0, v);
+        tmem_ld_wait(v);
+        const int q_cols = D % 64 == 0 ? 64 : min(D - c0, 64);
+        store_fragment(da, v, 0, fa, lane, q_cols, row0 + ra < p.seqlen, wide);
+        store_fragment(da + 8 * D, v, 2, fb, lane, q_cols, row0 + rb < p.seqlen, wide);
+      }
+    } else {
+      // Head dim 96: each thread its own row (half of the second fragment's
+      // lanes would have nothing to store).  4 x 4K, 55 heads: 308 us with
+      // fragments, 299 with rows (rolled 297, but 8K at block 64 108 -> 113);
+      // block 32, 2 x 4K, 32 heads: 201 -> 198; dense + mass 4K, 24 heads: 77.1
+      // -> 75.6.  Dense gains 2 % with query tiles paired and loses 1 % with
+      // heads paired, and keeps the fragments, as does head dim 128 (16K: 285 us
+      // with fragments, 294 with rows).
+#pragma unroll
+      for (int c0 = 0; c0 < D; c0 += 32) {
+        uint32_t v[32];
+        tmem_ld_32x32b_x32(o_col + c0, v);
+        tmem_ld_wait(v);
+        if (row < p.seqlen) {
+          __nv_bfloat16* dst = p.O + ((size_t)ent.y * p.seqlen + row) * D + c0;
+          const float2 f2 = make_float2(inv_l, inv_l);
+#pragma unroll
+          for (int c = 0; c < 32; c += 16) {
+            uint32_t q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const float2 x = __fmul2_rn(
+                  make_float2(__uint_as_float(v[c + 2 * k]), __uint_as_float(v[c + 2 * k + 1])), f2);
+              q[k] = pack_bf16x2(x.x, x.y);
+            }
+            store_16(dst + c, q, wide);
+          }
+        }
+      }
     }
   }
   // TMEM stores in flight complete before TMEM is released.
