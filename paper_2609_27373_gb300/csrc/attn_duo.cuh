@@ -43,15 +43,17 @@
 //   warp 12         stager: the units and, sparse, their tile masks
 //   warp 13         watchdog
 //
-// What bounds it (4K dense, 32 heads, head dim 128, a timeline of one CTA): a
-// stream's tile chain, 2830 clk for a tile of each stream against 2048 clk of
-// tensor work: S product 740 to its softmax's first load, load and row maximum
-// 440, exponentials and P 730 (550 of it the ex2 rate, 4.3 clk per warp
-// instruction), 450 until P V is issued, S(j+1) 440 behind it.  attn_kernel
-// takes 1930 clk a tile.  Measured against it (us, attn_kernel / here): dense
-// 119 / 105, dense + mass 128 / 112, sparse block 128 64 / 58, block 32 150 / 120;
-// 16K sparse 355 / 300; 32K, four heads to a kv head 850 / 705 (paired); 4 x 4K,
-// head dim 96 405 / 330.
+// What bounds it (a timeline of one CTA, head dim 128): a stream's tile chain,
+// 2830 clk for a tile of each stream against 2048 clk of tensor work: S product
+// 740 to its softmax's first load, load and row maximum 440, exponentials and P
+// 730 (550 of it the ex2 rate, 4.3 clk per warp instruction), 200 until the
+// issuing warp sees P, P V and S(j+1) behind one another.  attn_kernel takes
+// 1930 clk a tile.  A unit boundary costs a sparse stream 4400 clk more (16K, 11
+// tiles a unit): the diagonal's mask 600-1000, O's last product and the
+// epilogue 3100, the rest of the wait for the next unit's Q and first S.
+// Measured against attn_kernel (us, before / here): dense 120 / 102, dense + mass
+// 130 / 111, sparse block 128 64 / 57, block 32 150 / 110; 16K sparse 352 / 286; 32K,
+// four heads to a kv head 855 / 690 (paired); 4 x 4K, head dim 96 405 / 298.
 //
 // Every wait is bounded (the watchdog); a stream that stands still for the
 // launch's limit sets the status word and an abort flag, and every role unwinds.

@@ -141,18 +141,28 @@ bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long
 // With few units a CTA of the former has no second one to overlap with the
 // first, and a unit alone takes longer there.  Measured back to back in a graph
 // (us, attn_kernel / attn_duo_kernel; d = head dim, B = block):
-//   dense: 256 units (2K, 16 heads, d 128) 19.3 / 28.2, 384 (4K, 12 heads) 45.9 / 51.1,
-//     512 (4K, 16 heads) 55.9 / 51.7, 640 (4K, 20 heads) 70.2 / 64.2;
-//   sparse, B 128, d 128: 384 (4K) 26.6 / 28.2, 512 (4K) 31.9 / 32.0, 512 (8K) 41.0 /
-//     37.9, 640 (4K) 38.8 / 35.4; d 96: 768 43.7 / 40.2;
-//   sparse, smaller blocks: 192 (4K, d 128, B 64) 29.9 / 35.6, 512 (4K, d 128, B 64)
-//     61.9 / 52.4, 512 (2K, d 64, B 64) 36.5 / 29.2.
+//   dense: 256 units (2K, 16 heads, d 128) 19.4 / 27.4, 384 (4K, 12 heads) 46.3 / 49.1,
+//     512 (4K, 16 heads) 56.3 / 50.4, 640 (4K, 20 heads) 70.4 / 62.1;
+//   sparse, B 128, d 128: 384 (4K) 26.9 / 28.9, 512 (2K, 4 kv heads) 29.0 / 29.5, 512
+//     (4K) 32.0 / 32.0, 512 (8K) 41.2 / 37.7, 640 (4K) 39.1 / 34.9; d 96: 768 43.8 / 39.1;
+//   sparse, smaller blocks: 192 (4K, d 128, B 64) 30.3 / 35.8, 512 (4K, d 128, B 64)
+//     62.1 / 54.4, 512 (2K, d 64, B 64) 37.8 / 28.6.
+// Short sequences with 1.5 to 2 units per SM are the exception: it runs a CTA's
+// two units side by side, attn_kernel one after the other (attn_kernel's time
+// over this one's, sparse / dense / dense + mass, blocks of 32 to 128: 256 tokens,
+// d 64 to 128 1.01-1.22 / 1.01-1.19 / 1.17-1.44; 512 tokens, d 64 and 96 1.06-1.22 /
+// 1.00-1.11 / 1.15-1.28).  Not so with an odd number of query tiles, whose last
+// has no partner (dense, 384 tokens 0.86), 512 tokens at d 128 (dense 0.95), 1K
+// tokens (dense 0.79-0.91), or more than two units per SM (dense, 256 tokens
+// 0.85).
 // The line depends on the shape alone, not on the variant: sparse attention
 // over every block and dense attention run on the same kernel and give the
 // same bits.
-bool choose_duo(int mode, int sm_count, AttnParams& p) {
+bool choose_duo(int mode, int head_dim, int sm_count, AttnParams& p) {
   if (p.n_qtiles > 256) return false;  // the staged tile masks hold 256 key tiles
-  if (p.n_units < 3 * sm_count) return false;
+  const bool side_by_side = (p.n_qtiles == 2 || (p.n_qtiles == 4 && head_dim < 128)) &&
+                            2 * (long long)p.n_units >= 3 * sm_count && p.n_units <= 2 * sm_count;
+  if (p.n_units < 3 * sm_count && !side_by_side) return false;
   p.pair = kPairNone;
   p.v_heads = p.n_heads;
   p.v_qtiles = p.n_qtiles;
@@ -247,7 +257,7 @@ int launch_attention(const wise_shape_t* sh, const void* Q, const void* K, const
       if (!p.scratch) return WISE_ERR_CUDA;
     }
   }
-  const bool duo = choose_duo(mode, ds->sm_count, p);
+  const bool duo = choose_duo(mode, sh->head_dim, ds->sm_count, p);
   const int cols = duo ? duo_box_cols(sh->head_dim, p.pair != kPairNone) : 64;
   if (!make_map(&L.mapQ, Q, sh->head_dim, sh->seqlen, outer_q, 128, cols) ||
       !make_map(&L.mapK, K, sh->head_dim, sh->seqlen, outer_kv, 128, cols) ||

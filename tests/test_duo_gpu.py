@@ -1,7 +1,8 @@
 """The two-stream attention kernel (attn_duo.cuh), which launches with several
 query tiles per SM take: dense, dense + mass and sparse against the oracle at
 the sizes where its pairing, tile and schedule code can go wrong.  Every shape
-here has at least 4 x 152 query tiles, so that it runs on any GB300.
+here has at least 4 x 152 query tiles, so that it runs on any GB300, or is a
+short sequence with 1.5 to 2 query tiles per SM.
 
 Tolerances are those of the parity tests (gpu_helpers)."""
 import numpy as np
@@ -22,6 +23,7 @@ SHAPES = [
     (4, 52, 52, 384, 128, 128), (2, 40, 40, 1024, 128, 128), (4, 33, 11, 640, 128, 128), (4, 64, 16, 384, 128, 128),
     (4, 55, 55, 384, 96, 128), (3, 54, 9, 544, 96, 32), (4, 40, 40, 576, 64, 64), (4, 64, 32, 416, 64, 32),
     (8, 80, 80, 128, 64, 128), (10, 64, 8, 96, 64, 32), (2, 37, 37, 1120, 96, 32),
+    (1, 125, 125, 256, 128, 128), (2, 36, 36, 416, 64, 32), (4, 16, 16, 512, 96, 64), (3, 40, 8, 160, 128, 32),
 ]
 
 
