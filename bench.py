@@ -62,7 +62,7 @@ def sparse_traffic_bytes():
     """DRAM bytes per launch of the sparse kernel from the committed ncu
     summary, or None when the kernel source changed since that capture."""
     import hashlib
-    src = os.path.join(ROOT, "paper_2609_27373_gb300", "csrc", "attn_kernel.cuh")
+    src = os.path.join(ROOT, "paper_2609_27373_gb300", "csrc", "attn_duo.cuh")
     prof = os.path.join(ROOT, "profiles", "attn_sparse_4k.md")
     try:
         sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
