@@ -196,13 +196,12 @@ __device__ __forceinline__ bool duo_warp_wait(uint64_t* bar, uint32_t parity, co
   return __all_sync(0xffffffffu, duo_wait(bar, parity, abort));
 }
 
-// On the way out: a wait for work in flight, with its own limit (the SM clock
-// is 2.07 GHz at most, so 2 clk are at least 1 ns).
+// On the way out: a wait for work in flight, with its own limit.
 __device__ __forceinline__ void duo_drain(uint64_t* bar, uint32_t parity) {
-  const long long t0 = clock64();
+  const uint64_t t0 = global_timer_ns();
 #pragma unroll 1
   while (!mbar_try_wait(bar, parity))
-    if (clock64() - t0 > (long long)(2 * kWaitLimitNs)) return;
+    if (global_timer_ns() - t0 > kWaitLimitNs) return;
 }
 
 // Warp 13, one lane: every wait of a stream's tile chain ends in time as long
@@ -211,20 +210,20 @@ template <class Sh>
 __device__ void duo_watchdog(const AttnParams& p, Sh& sb) {
   volatile int* beat = sb.beat;
   int last0 = 0, last1 = 0;
-  long long t0 = clock64(), t1 = t0;
+  uint64_t t0 = global_timer_ns(), t1 = t0;
 #pragma unroll 1
   for (uint32_t it = 0;; ++it) {
     const bool d0 = mbar_test_wait(&sb.done[0], 0);
     if (d0 && mbar_try_wait(&sb.done[1], 0)) return;
     if (!d0 && mbar_try_wait(&sb.done[0], 0)) continue;
     const int b0 = beat[0], b1 = beat[1];
-    const long long now = clock64();
+    const uint64_t now = global_timer_ns();
     if (d0 || b0 != last0) t0 = now;
     if (b1 != last1 || mbar_test_wait(&sb.done[1], 0)) t1 = now;
     last0 = b0;
     last1 = b1;
-    const long long limit = (long long)(2 * p.wait_ns);
-    if (now - t0 > limit || now - t1 > limit) {
+    // Unsigned, like mbar_wait: the limit may be any 64-bit number.
+    if (now - t0 > p.wait_ns || now - t1 > p.wait_ns) {
       raise_status(p, &sb.abort, kStatusTimeout);
       return;
     }
