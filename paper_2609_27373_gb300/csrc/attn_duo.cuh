@@ -145,7 +145,7 @@ struct DuoShared {
   typename std::conditional<MODE == kDenseMass, DuoMassSums, DuoNoMass>::type mass;
   uint32_t tmem_base;
   int abort;
-  int beat[2];  // tiles begun by each stream
+  int beat[2];  // per stream, by its softmax: twice the entries taken, less one while it works on the last of them
 };
 
 // Unit u -> (batch, virtual head, virtual query tile): see decode_unit; a
@@ -177,12 +177,12 @@ __device__ __forceinline__ bool duo_unit(const AttnParams& p, int k, int& u) {
 }
 
 // Waits end when the phase completes or the abort flag is set; the watchdog
-// (warp 13) sets the flag when a stream makes no progress for the launch's
-// limit.  Code size matters in this kernel: its roles together run more
-// instructions than the SM's instruction cache holds, and with a timed loop at
-// every wait and everything unrolled (99 KB) a fifth of the fetches missed and
-// the warps stalled 1.6 cycles per instruction for instructions; hence also
-// the rolled loops on whatever is not the tile loop.
+// (warp 13) sets the flag when a stream stands still for the launch's limit.
+// Code size matters in this kernel: its roles together run more instructions
+// than the SM's instruction cache holds, and with a timed loop at every wait
+// and everything unrolled (99 KB) a fifth of the fetches missed and the warps
+// stalled 1.6 cycles per instruction for instructions; hence also the rolled
+// loops on whatever is not the tile loop.
 __device__ __forceinline__ bool duo_wait(uint64_t* bar, uint32_t parity, const volatile int* abort) {
   const uint32_t at = smem_u32(bar);
 #pragma unroll 1
@@ -204,8 +204,12 @@ __device__ __forceinline__ void duo_drain(uint64_t* bar, uint32_t parity) {
     if (global_timer_ns() - t0 > kWaitLimitNs) return;
 }
 
-// Warp 13, one lane: every wait of a stream's tile chain ends in time as long
-// as the stream's tile counter moves.
+// Warp 13, one lane.  A stream's clock runs from the moment its softmax takes a
+// schedule entry until it is ready for the next one (a key tile, the unit's
+// epilogue with its last).  A stream that waits for an entry has nothing to do
+// as long as the other one moves: a paired unit may hold tiles for one stream
+// only, and a stream may run out of units early.  Both standing still, working
+// or not, is a wait of the producers or the stager that does not end.
 template <class Sh>
 __device__ void duo_watchdog(const AttnParams& p, Sh& sb) {
   volatile int* beat = sb.beat;
@@ -217,13 +221,15 @@ __device__ void duo_watchdog(const AttnParams& p, Sh& sb) {
     if (d0 && mbar_try_wait(&sb.done[1], 0)) return;
     if (!d0 && mbar_try_wait(&sb.done[0], 0)) continue;
     const int b0 = beat[0], b1 = beat[1];
+    const bool d1 = mbar_test_wait(&sb.done[1], 0);
     const uint64_t now = global_timer_ns();
-    if (d0 || b0 != last0) t0 = now;
-    if (b1 != last1 || mbar_test_wait(&sb.done[1], 0)) t1 = now;
+    if (b0 != last0) t0 = now;
+    if (b1 != last1) t1 = now;
     last0 = b0;
     last1 = b1;
     // Unsigned, like mbar_wait: the limit may be any 64-bit number.
-    if (now - t0 > p.wait_ns || now - t1 > p.wait_ns) {
+    const uint64_t both = max(t0, t1);
+    if ((!d0 && now - ((b0 & 1) ? t0 : both) > p.wait_ns) || (!d1 && now - ((b1 & 1) ? t1 : both) > p.wait_ns)) {
       raise_status(p, &sb.abort, kStatusTimeout);
       return;
     }
@@ -656,7 +662,6 @@ __device__ void duo_mma(const CUtensorMap* mapQ, const AttnParams& p, int s, uin
         umma_commit(&sb.empty[k_slot]);
         if (ent.z & kEntSolo) umma_commit(&sb.empty[k_slot]);
       }
-      sb.beat[s] = pos;
     };
     if (due) {
       const uint32_t acc = (fl & kEntFirst) ? 0u : 1u;
@@ -879,6 +884,7 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
 
   for (;;) {
     const int slot = pos % kDuoSlots;
+    if (r == 0) sb.beat[w] = 2 * pos;
     if (!duo_warp_wait(&sb.sched_full[w][slot], (pos / kDuoSlots) & 1, abort)) {
       ok = false;
       break;
@@ -887,6 +893,7 @@ __device__ void duo_softmax(const AttnParams& p, int w, uint32_t tmem, Sh& sb) {
     __syncwarp();
     if (lane == 0) mbar_arrive(&sb.sched_empty[w][slot]);
     ++pos;
+    if (r == 0) sb.beat[w] = 2 * pos - 1;
     if (ent.z & kEntEnd) break;
     const int qt = ent.w >> 16, t = ent.w & 0xFFFF;
     const int row = qt * 128 + r;
