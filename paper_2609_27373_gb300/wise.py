@@ -148,8 +148,17 @@ def _ptr(t):
 
 
 @functools.lru_cache(maxsize=256)
+def _struct(value):
+    return value, ctypes.byref(value.c())
+
+
 def _c(value):
     """Reference to the C struct of a Shape or Select (read only)."""
+    first, ref = _struct(value)
+    # 8.0 equals 8, but no int field takes it: an equal value of other types
+    # goes through the conversion itself.
+    if first is value or [*map(type, vars(first).values())] == [*map(type, vars(value).values())]:
+        return ref
     return ctypes.byref(value.c())
 
 
