@@ -240,10 +240,13 @@ __device__ void duo_watchdog(const AttnParams& p, Sh& sb) {
 // ------------------------------------------------------------------- stager
 // Warp 12: the CTA's units in order and, sparse, the masks of their key tiles
 // from their S support lists.  An entry of list q is accepted if it lies in
-// [0, q0 + q] and exceeds every in-range entry before it (TileIter's rule); a
-// warp prefix max over 32 entries at a time decides that for all of them at
-// once, the next 32 being loaded meanwhile.  After the last unit come two end
-// markers, one for each producer.
+// [0, q0 + q] and exceeds every in-range entry before it (TileIter's rule).  32
+// entries are judged at a time, the next 32 being loaded meanwhile: each above
+// its neighbour, as in a list that is as it should be, or by a warp prefix max.
+// Units of few tiles are bound by this warp.  Lists of three entries at block 32
+// (us, every row walked to its end with a prefix max for all / here): 16K,
+// 32 heads, rows of 32 171 / 173, rows of 512 954 / 174; 32K, 8 heads, rows of
+// 1024 971 / 97.  After the last unit come two end markers, one for each producer.
 template <int D, int BLK, int MODE, class Sh>
 __device__ void duo_stager(const AttnParams& p, Sh& sb) {
   constexpr int S = kTileN / BLK;
@@ -251,7 +254,6 @@ __device__ void duo_stager(const AttnParams& p, Sh& sb) {
   auto& st = sb.stage;
   const int lane = threadIdx.x & 31;
   volatile int* abort = &sb.abort;
-  const int chunks = (p.cap + 31) / 32;  // of one list
   int bad = 0, ends = 0;
   bool ok = true;
   for (int k = 0, n_st = 0; ends < 2; ++k) {
@@ -281,14 +283,18 @@ __device__ void duo_stager(const AttnParams& p, Sh& sb) {
         for (int i = lane; i < n_words; i += 32) st.mask[slot][i] = 0u;
         __syncwarp();
         const size_t row0 = (size_t)z * p.n_blocks + q0;
-        const int32_t* counts = p.counts + row0;
         const int32_t* list = p.idx + row0 * p.cap;
+        const int32_t* counts = p.counts + row0;
         int q = 0, x = 0, carry = -1;  // list, first entry
         int cnt = __ldg(counts);
         int v = lane < p.cap ? __ldg(list + lane) : -1;
 #pragma unroll 1
-        for (int c = 0; c < n_lists * chunks; ++c) {
-          const int nx = x + 32 < p.cap ? x + 32 : 0, nq = nx == 0 ? q + 1 : q;
+        while (q < n_lists) {
+          // A list is read as far as its count goes.  In rows of up to 32 the next
+          // load need not wait for the count: the next list follows in any case.
+          bool more_of = false;
+          if (p.cap > 32) more_of = x + 32 < clamp_count(cnt, p.cap, bad);
+          const int nx = more_of ? x + 32 : 0, nq = more_of ? q : q + 1;
           int n_cnt = 0, n_v = -1;
           if (nq < n_lists) {
             n_cnt = __ldg(counts + nq);
@@ -298,16 +304,25 @@ __device__ void duo_stager(const AttnParams& p, Sh& sb) {
           const bool live = x + lane < clamp_count(cnt, p.cap, bad);
           const bool in_range = live && v >= 0 && v <= q0 + q;
           int m = in_range ? v : -1;
-#pragma unroll 1
-          for (int o = 1; o < 32; o <<= 1) {
-            const int other = __shfl_up_sync(0xffffffffu, m, o);
-            if (lane >= o) m = max(m, other);
-          }
           int before = __shfl_up_sync(0xffffffffu, m, 1);
-          before = max(lane == 0 ? -1 : before, carry);
-          const bool acc = in_range && v > before;
-          if (live && !acc) bad = 1;
-          carry = max(carry, __shfl_sync(0xffffffffu, m, 31));
+          if (lane == 0) before = carry;
+          const unsigned lanes = __ballot_sync(0xffffffffu, live);
+          bool acc = in_range && m > before;
+          if (__ballot_sync(0xffffffffu, acc) != lanes) {
+            // Something not ascending or out of range: a prefix maximum decides.
+#pragma unroll 1
+            for (int o = 1; o < 32; o <<= 1) {
+              const int other = __shfl_up_sync(0xffffffffu, m, o);
+              if (lane >= o) m = max(m, other);
+            }
+            before = __shfl_up_sync(0xffffffffu, m, 1);
+            before = max(lane == 0 ? -1 : before, carry);
+            acc = in_range && v > before;
+            bad = 1;
+            carry = max(carry, __shfl_sync(0xffffffffu, m, 31));
+          } else if (lanes) {
+            carry = __shfl_sync(0xffffffffu, m, 31 - __clz(lanes));
+          }
           if (acc) {
             const int bit = (v / S) * (S * S) + q * S + v % S;
             atomicOr(&st.mask[slot][bit >> 5], 1u << (bit & 31));
