@@ -17,7 +17,9 @@
 //               query tile: the same key tiles, so each K and V tile is loaded
 //               once for both.
 //   kPairTiles  (dense variants) stream s takes query tile 2 v + s of the same
-//               head: K and V tiles shared up to the diagonal.
+//               head, less AttnParams::lone_first: K and V tiles shared up to the
+//               diagonal.  Of an odd number of tiles the last, or the first, has
+//               no partner and leaves one stream without work.
 //
 // Tensor memory (512 columns): S of stream s at 128 s, with P (bf16 pairs)
 // written over its first 64 columns, and O of stream s at 256 + 128 s.
@@ -272,10 +274,11 @@ __device__ void duo_stager(const AttnParams& p, Sh& sb) {
     }
     const int h = p.pair == kPairHeads ? 2 * vh : vh;
     const int z = b * p.n_kv_heads + h / p.group;
+    const int qt = p.pair == kPairTiles ? 2 * vq - p.lone_first : vq;  // of stream 0 (-1: stream 1 alone)
     int n = -1;
     if (more) {
       if constexpr (MODE != kSparse) {
-        n = (p.pair == kPairTiles ? min(2 * vq + 1, p.n_qtiles - 1) : vq) + 1;
+        n = (p.pair == kPairTiles ? min(qt + 1, p.n_qtiles - 1) : qt) + 1;
       } else {
         const int q0 = vq * S;
         const int n_lists = min(S, p.n_blocks - q0);
@@ -344,7 +347,7 @@ __device__ void duo_stager(const AttnParams& p, Sh& sb) {
       }
     }
     if (lane == 0) {
-      st.unit[slot] = make_int4(n, b * p.n_heads + h, z, p.pair == kPairTiles ? 2 * vq : vq);
+      st.unit[slot] = make_int4(n, b * p.n_heads + h, z, qt);
       mbar_arrive(&st.full[slot]);
     }
     ++n_st;
@@ -531,10 +534,10 @@ __device__ void duo_producer_paired(const CUtensorMap* mapK, const CUtensorMap* 
     }
     if (lane == 0) {
       const int bh1 = unit.y + (heads ? 1 : 0), qt1 = heads ? unit.w : unit.w + 1;
-      const bool two = qt1 < p.n_qtiles;  // an odd last query tile goes to stream 0 alone
-      if (unit.x <= 0) {
+      const bool two = qt1 < p.n_qtiles;  // not the last of an odd number of query tiles
+      if (unit.x <= 0) {  // no tile (sparse, head pairs), or the end
         const int fl = unit.x < 0 ? kEntEnd : kEntEmpty;
-        ok = duo_emit(p, 0, pos0, make_int4(0, unit.y, fl, unit.w << 16), sb) &&
+        ok = duo_emit(p, 0, pos0, make_int4(0, unit.y, fl, qt1 << 16), sb) &&
              duo_emit(p, 1, pos1, make_int4(0, bh1, fl, qt1 << 16), sb);
       }
       DuoWalk<BLK, MODE> walk;
@@ -542,7 +545,7 @@ __device__ void duo_producer_paired(const CUtensorMap* mapK, const CUtensorMap* 
       for (int t = 0; t < unit.x; ++t, ++n) {
         const uint32_t key = walk.next(sb.stage.taken[0]);
         const int kt = (int)(key & 0xFFFFu);
-        // kPairTiles: stream 0 ends one tile before stream 1.
+        // kPairTiles: stream 0 ends one tile before stream 1, or has none.
         const bool use0 = heads || kt <= unit.w;
         const int last = t + 1 == unit.x ? kEntLast : 0;
         const int fl = (n << 8) | (t == 0 ? kEntFirst : 0) | (use0 && two ? 0 : kEntSolo);

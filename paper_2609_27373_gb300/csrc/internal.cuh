@@ -49,6 +49,7 @@ struct AttnParams {
   // attn_duo_kernel: the pairing, and its units (virtual heads and query
   // tiles, see decode_duo).
   int pair, v_heads, v_qtiles, v_units, v_group_heads;
+  int lone_first;  // kPairTiles, odd number of query tiles: 1 if the first one has no partner, 0 if the last
   int o_align32;  // O is 32-byte aligned
 };
 

@@ -164,6 +164,7 @@ bool choose_duo(int mode, int head_dim, int sm_count, AttnParams& p) {
                             2 * (long long)p.n_units >= 3 * sm_count && p.n_units <= 2 * sm_count;
   if (p.n_units < 3 * sm_count && !side_by_side) return false;
   p.pair = kPairNone;
+  p.lone_first = 0;
   p.v_heads = p.n_heads;
   p.v_qtiles = p.n_qtiles;
   p.v_group_heads = p.group_heads;
@@ -173,8 +174,16 @@ bool choose_duo(int mode, int head_dim, int sm_count, AttnParams& p) {
     p.v_heads = p.n_heads / 2;
     p.v_group_heads = p.group_heads / 2;
   } else if (mode != kSparse) {
+    // Of an odd number of tiles one has no partner, and its unit leaves one
+    // stream idle.  Up to 4 units per SM the last and longest one is then the
+    // launch's time, and the first takes its place (us, last alone / first alone /
+    // attn_kernel, dense, d 128: 92 heads x 640 tokens 20.8 / 17.0 / 18.2, 66 x 896
+    // 22.7 / 20.1 / 20.4, d 64 mass 92 x 640 17.0 / 14.5 / 19.4).  Beyond that it depends on how the units fall (198 x 640 33.6 /
+    // 30.9, 244 x 640 42.0 / 43.0, batch 2, 24 x 2944 97.4 / 105.3); three tiles
+    // have too little after the pair (203 x 384 17.0 / 18.6).
     p.pair = kPairTiles;
     p.v_qtiles = (p.n_qtiles + 1) / 2;
+    p.lone_first = p.n_qtiles % 2 != 0 && p.n_qtiles >= 5 && p.n_units <= 4 * sm_count;
   }
   p.v_units = p.batch * p.v_heads * p.v_qtiles;
   return true;
