@@ -157,12 +157,17 @@ bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long
 // 0.85).
 // The line depends on the shape alone, not on the variant: sparse attention
 // over every block and dense attention run on the same kernel and give the
-// same bits.
+// same bits.  One query tile is the exception: a unit of one key tile comes out
+// the same on either, and dense without head pairs would leave the second stream
+// idle (attn_kernel / attn_duo_kernel, 912 heads x 128 tokens, d 64, 96, 128: dense
+// 14.1 / 15.1, 17.5 / 19.4, 22.2 / 24.6; dense + mass 24.0 / 18.4, 26.7 / 19.1, 30.4 /
+// 26.0, sparse, unpaired, 17.0 / 13.9, 18.7 / 15.5, 23.6 / 21.4).
 bool choose_duo(int mode, int head_dim, int sm_count, AttnParams& p) {
   if (p.n_qtiles > 256) return false;  // the staged tile masks hold 256 key tiles
   const bool side_by_side = (p.n_qtiles == 2 || (p.n_qtiles == 4 && head_dim < 128)) &&
                             2 * (long long)p.n_units >= 3 * sm_count && p.n_units <= 2 * sm_count;
   if (p.n_units < 3 * sm_count && !side_by_side) return false;
+  if (mode == kDense && p.n_qtiles == 1 && p.group % 2 != 0) return false;
   p.pair = kPairNone;
   p.lone_first = 0;
   p.v_heads = p.n_heads;
@@ -178,9 +183,10 @@ bool choose_duo(int mode, int head_dim, int sm_count, AttnParams& p) {
     // stream idle.  Up to 4 units per SM the last and longest one is then the
     // launch's time, and the first takes its place (us, last alone / first alone /
     // attn_kernel, dense, d 128: 92 heads x 640 tokens 20.8 / 17.0 / 18.2, 66 x 896
-    // 22.7 / 20.1 / 20.4, d 64 mass 92 x 640 17.0 / 14.5 / 19.4).  Beyond that it depends on how the units fall (198 x 640 33.6 /
-    // 30.9, 244 x 640 42.0 / 43.0, batch 2, 24 x 2944 97.4 / 105.3); three tiles
-    // have too little after the pair (203 x 384 17.0 / 18.6).
+    // 22.7 / 20.1 / 20.4, d 64 mass 92 x 640 17.0 / 14.5 / 19.4).  Beyond that it
+    // depends on how the units fall (198 x 640 33.6 / 30.9, 244 x 640 42.0 / 43.0,
+    // batch 2, 24 x 2944 97.4 / 105.3); three tiles have too little after the
+    // pair (203 x 384 17.0 / 18.6).
     p.pair = kPairTiles;
     p.v_qtiles = (p.n_qtiles + 1) / 2;
     p.lone_first = p.n_qtiles % 2 != 0 && p.n_qtiles >= 5 && p.n_units <= 4 * sm_count;
