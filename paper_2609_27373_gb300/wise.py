@@ -147,19 +147,20 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
-@functools.lru_cache(maxsize=256)
-def _struct(value):
-    return value, ctypes.byref(value.c())
+# By the types of the fields too: 8.0 equals 8, but no int field takes it.
+@functools.lru_cache(maxsize=256, typed=True)
+def _struct(cls, *fields):
+    return ctypes.byref(cls(*fields).c())
 
 
-def _c(value):
-    """Reference to the C struct of a Shape or Select (read only)."""
-    first, ref = _struct(value)
-    # 8.0 equals 8, but no int field takes it: an equal value of other types
-    # goes through the conversion itself.
-    if first is value or [*map(type, vars(first).values())] == [*map(type, vars(value).values())]:
-        return ref
-    return ctypes.byref(value.c())
+def _c(s):
+    """Reference to the C struct of a Shape (read only)."""
+    return _struct(Shape, s.batch, s.seqlen, s.n_heads, s.n_kv_heads, s.head_dim, s.block, s.scale)
+
+
+def _c_select(s):
+    """Reference to the C struct of a Select (read only)."""
+    return _struct(Select, s.n_sink, s.n_local, s.mode, s.topk, s.eta, s.cap)
 
 
 def _check(t, name, shape, dtype):
@@ -222,7 +223,7 @@ def wise_select_support(shape: Shape, sel: Select, blockmass, idx, counts, strea
     _check(blockmass, "blockmass", (shape.batch, shape.n_heads, nb, nb), torch.float32)
     _check(idx, "idx", (shape.batch, shape.n_kv_heads, nb, sel.cap), torch.int32)
     _check(counts, "counts", (shape.batch, shape.n_kv_heads, nb), torch.int32)
-    rc = load().wise_select_support(_c(shape), _c(sel), _ptr(blockmass), _ptr(idx), _ptr(counts),
+    rc = load().wise_select_support(_c(shape), _c_select(sel), _ptr(blockmass), _ptr(idx), _ptr(counts),
                                     _stream(stream))
     if rc != WISE_OK:
         raise WiseError(rc, "wise_select_support")
