@@ -15,13 +15,19 @@
 // The fixed-point conversion is integer arithmetic, not double precision, whose
 // rate on this chip is 1/64 of single precision's, and reductions use the warp
 // reduction instructions.  Ranking (take_ranked) depends on the row: up to 32
-// blocks are compared all with all, few picks are taken one by one, and many by
-// a binary search for the mass of the last pick.  Measured back to back in a
-// graph (us, with double precision, one-by-one picks and shuffles / here): 32K,
-// 4 heads per kv head, top 12: 22.6 / 12.8; coverage up to 32 of 128 blocks 32.8 /
-// 18.0; working sets of 4 steps: 4K 40 / 8.6, 16K (128 blocks) 316 / 58, 32K (5
-// steps) 734 / 84.
+// blocks are compared all with all; otherwise picks are taken one by one, and
+// where four do not suffice and many may follow, a search over the mass of the
+// last pick narrows the rest down to a few.  Measured back to back in a graph
+// (us, with double precision, one-by-one picks and shuffles / here): 32K, 4 heads
+// per kv head, top 12 22.6 / 12.8; 32 heads of 128 blocks, masses a softmax of
+// normals, coverage up to 32 blocks: std 1 33.6 / 10.7, std 12 (one block holds most
+// of a row) 8.9 / 6.0; working sets of two steps: std 1 160 / 21, std 12 13.0 / 8.5;
+// of 256 blocks 575 / 53, 31 / 20; 4 heads of 1024 blocks 2560 / 131, 91 / 52.
+// With the search from the first pick on, down to the last bit, concentrated
+// rows were bound by it: the cases at std 12 took 19.6, 32.7, 84 and 151.
 #include <limits.h>
+
+#include <algorithm>
 
 #include "internal.cuh"
 
@@ -60,11 +66,20 @@ __device__ __forceinline__ bool below_threshold(uint64_t cum, uint64_t eta16, ui
   return lhs_hi < rhs_hi || (lhs_hi == rhs_hi && lhs_lo < rhs_lo);
 }
 
+// Rows that may take up to kFewPicks blocks take them one by one.  In the others
+// the search follows kFirstPicks picks (2 and 0 were slower on concentrated rows,
+// 128 blocks, std 12: 8.5 / 9.9 / 12.8 us) and ends when kLeft blocks are undecided
+// (2 and 8 within 3 %).  A launch in which no row may take more has an instance
+// without the search: its registers cost top 8 of 256 blocks 13.7 -> 14.2 us.
+constexpr int kFewPicks = 16;
+constexpr int kFirstPicks = 4;
+constexpr int kLeft = 4;
+
 // Adds candidates in rank order to `chosen` until done(kept mass, number
 // added), which stays true once it is true; `cum` is the mass kept before, and
 // `most` an upper bound on the number added.  Bit i of cand / chosen is block
 // lane + 32 i.
-template <int KPL, class Done>
+template <int KPL, bool kFew, class Done>
 __device__ __forceinline__ void take_ranked(const uint64_t (&U)[KPL], uint32_t cand, uint32_t& chosen, uint64_t cum,
                                             int most, int lane, Done done) {
   if (done(cum, 0)) return;
@@ -84,55 +99,80 @@ __device__ __forceinline__ void take_ranked(const uint64_t (&U)[KPL], uint32_t c
     }
     if (cand && !done(cum + before, rank)) chosen |= 1u;
   } else {
+    // One at a time: the largest mass, then the lowest block.
     int added = 0;
-    if (most > 16) {
-      // The largest T such that the blocks of mass >= T suffice, bit by bit.
-      uint64_t top = 0, part = 0;
-#pragma unroll
-      for (int i = 0; i < KPL; ++i) {
-        if ((cand >> i) & 1u) {
-          top = max(top, U[i]);
-          part += U[i];
-        }
-      }
-      if (!done(cum + warp_sum_u64(part), __reduce_add_sync(0xffffffffu, __popc(cand)))) {
-        chosen |= cand;  // all of them do not suffice
-        return;
-      }
-      top = warp_max_u64(top);
-      uint64_t T = 0;
-      for (int bit = 63 - __clzll((long long)(top | 1ull)); bit >= 0; --bit) {
-        const uint64_t t = T | (1ull << bit);
-        uint64_t s = 0;
-        int n = 0;
+    for (int first = !kFew && most > kFewPicks ? kFirstPicks : INT_MAX;; --first) {
+      if (!kFew && first == 0) {
+        // Masses lo and hi such that the blocks of mass >= lo suffice and those of
+        // mass >= hi do not, closed in bit by bit until few blocks lie between.
+        uint64_t top = 0, part = 0;
 #pragma unroll
         for (int i = 0; i < KPL; ++i) {
-          const bool in = ((cand >> i) & 1u) && U[i] >= t;
-          s += in ? U[i] : 0ull;
-          n += in;
+          if ((cand >> i) & 1u) {
+            top = max(top, U[i]);
+            part += U[i];
+          }
         }
-        if (done(cum + warp_sum_u64(s), __reduce_add_sync(0xffffffffu, n))) T = t;
-      }
-      // Every block above T; those of mass T one by one below.
-      uint64_t s = 0;
-      uint32_t above = 0, equal = 0;
+        int n_lo = __reduce_add_sync(0xffffffffu, __popc(cand)), n_hi = 0;  // blocks of mass >= lo, >= hi
+        if (!done(cum + warp_sum_u64(part), added + n_lo)) {
+          chosen |= cand;  // all of them do not suffice
+          return;
+        }
+        top = warp_max_u64(top);
+        uint64_t lo = 0, hi = ~0ull, s_hi = 0;
+        for (int bit = 63 - __clzll((long long)(top | 1ull)); bit >= 0 && n_lo - n_hi > kLeft; --bit) {
+          const uint64_t t = lo | (1ull << bit);
+          uint64_t s = 0;
+          int n = 0;
 #pragma unroll
-      for (int i = 0; i < KPL; ++i) {
-        if (!((cand >> i) & 1u)) continue;
-        if (U[i] > T) {
-          above |= 1u << i;
-          s += U[i];
-        } else if (U[i] == T) {
-          equal |= 1u << i;
+          for (int i = 0; i < KPL; ++i) {
+            const bool in = ((cand >> i) & 1u) && U[i] >= t;
+            s += in ? U[i] : 0ull;
+            n += in;
+          }
+          s = warp_sum_u64(s);
+          n = __reduce_add_sync(0xffffffffu, n);
+          if (done(cum + s, added + n)) {
+            lo = t;
+            n_lo = n;
+          } else {
+            hi = t;
+            n_hi = n;
+            s_hi = s;
+          }
+        }
+        // The blocks of mass >= hi, and of those between one by one below.
+        uint32_t above = 0, between = 0;
+#pragma unroll
+        for (int i = 0; i < KPL; ++i) {
+          if (!((cand >> i) & 1u)) continue;
+          if (U[i] >= hi) {
+            above |= 1u << i;
+          } else if (U[i] >= lo) {
+            between |= 1u << i;
+          }
+        }
+        chosen |= above;
+        cum += s_hi;
+        added += n_hi;
+        cand = between;
+        const int n_eq = n_lo - n_hi;
+        if (n_eq > kLeft) {
+          // No bit is left: all of them have mass lo.  The fewest that suffice,
+          // the lowest blocks first.
+          int take = 0;
+          for (int step = 1 << (31 - __clz(n_eq)); step > 0; step >>= 1)
+            if (take + step <= n_eq && !done(cum + (uint64_t)(take + step) * lo, added + take + step)) take += step;
+          ++take;
+#pragma unroll
+          for (int i = 0; i < KPL; ++i) {
+            const uint32_t ball = __ballot_sync(0xffffffffu, (between >> i) & 1u);
+            if (((between >> i) & 1u) && __popc(ball & ((1u << lane) - 1u)) < take) chosen |= 1u << i;
+            take -= __popc(ball);
+          }
+          return;
         }
       }
-      chosen |= above;
-      cum += warp_sum_u64(s);
-      added = __reduce_add_sync(0xffffffffu, __popc(above));
-      cand = equal;
-    }
-    // One at a time: the largest mass, then the lowest block.
-    while (!done(cum, added)) {
       uint64_t best_u = 0;
       int best_kb = INT_MAX;
 #pragma unroll
@@ -151,6 +191,7 @@ __device__ __forceinline__ void take_ranked(const uint64_t (&U)[KPL], uint32_t c
       }
       cum += u;
       ++added;
+      if (done(cum, added)) return;
     }
   }
 }
@@ -189,7 +230,7 @@ __device__ __forceinline__ void write_row(uint32_t chosen, int32_t* out, int cap
   if (lane == 0) *count = n;
 }
 
-template <int KPL>
+template <int KPL, bool kFew>
 __global__ void __launch_bounds__(256) select_kernel(const SelectParams p) {
   const long row = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long n_rows = (long)p.batch * p.n_kv_heads * p.n_blocks;
@@ -223,7 +264,7 @@ __global__ void __launch_bounds__(256) select_kernel(const SelectParams p) {
   const int n_forced = __reduce_add_sync(0xffffffffu, __popc(chosen));
   const int budget = (p.mode == 0) ? min(p.topk, p.cap - n_forced) : p.cap - n_forced;
   const bool coverage = p.mode != 0;
-  take_ranked(U, cand, chosen, cum, budget, lane, [&](uint64_t c, int n) {
+  take_ranked<KPL, kFew>(U, cand, chosen, cum, budget, lane, [&](uint64_t c, int n) {
     return n >= budget || (coverage && !below_threshold(c, p.eta16, total));
   });
   write_row<KPL>(chosen, p.idx + row * p.cap, p.cap, p.counts + row, lane);
@@ -234,7 +275,11 @@ static cudaError_t launch_select_kpl(const SelectParams& p, cudaStream_t stream)
   const long rows = (long)p.batch * p.n_kv_heads * p.n_blocks;
   const int warps = 8;
   const long grid = (rows + warps - 1) / warps;
-  select_kernel<KPL><<<(unsigned)grid, warps * 32, 0, stream>>>(p);
+  const int most = p.mode == 0 ? std::min(p.topk, p.cap) : p.cap;
+  if (KPL > 1 && most <= kFewPicks)
+    select_kernel<KPL, true><<<(unsigned)grid, warps * 32, 0, stream>>>(p);
+  else
+    select_kernel<KPL, false><<<(unsigned)grid, warps * 32, 0, stream>>>(p);
   return cudaGetLastError();
 }
 
@@ -256,8 +301,9 @@ cudaError_t launch_select(const SelectParams& p, cudaStream_t stream) {
 // 2 mass matched, 3 size matched (first step's ranking against a reference
 // working set).  Forced sink/local blocks belong to every set.
 
+// Two CTAs per SM at 32 blocks a lane (1024 blocks, std 12: 67 -> 52 us).
 template <int KPL>
-__global__ void __launch_bounds__(256) working_set_kernel(const WorkingSetParams p) {
+__global__ void __launch_bounds__(256, KPL >= 32 ? 2 : 0) working_set_kernel(const WorkingSetParams p) {
   const long row = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long n_rows = (long)p.batch * p.n_kv_heads * p.n_blocks;
   if (row >= n_rows) return;
@@ -291,7 +337,7 @@ __global__ void __launch_bounds__(256) working_set_kernel(const WorkingSetParams
       }
       const uint64_t total = warp_sum_u64(total_part);
       uint32_t chosen = forced;
-      take_ranked(U, admissible & ~forced, chosen, warp_sum_u64(cum_part), nb, lane,
+      take_ranked<KPL, false>(U, admissible & ~forced, chosen, warp_sum_u64(cum_part), nb, lane,
                   [&](uint64_t c, int) { return !below_threshold(c, p.eta16, total); });
       result |= chosen;
     }
@@ -333,9 +379,9 @@ __global__ void __launch_bounds__(256) working_set_kernel(const WorkingSetParams
     const int k_more = k_ref - __reduce_add_sync(0xffffffffu, n_forced_part);
     uint32_t chosen = forced;
     if (p.mode == 2)
-      take_ranked(U, admissible & ~forced, chosen, cum, nb, lane, [&](uint64_t c, int) { return c >= target; });
+      take_ranked<KPL, false>(U, admissible & ~forced, chosen, cum, nb, lane, [&](uint64_t c, int) { return c >= target; });
     else
-      take_ranked(U, admissible & ~forced, chosen, cum, k_more, lane, [&](uint64_t, int n) { return n >= k_more; });
+      take_ranked<KPL, false>(U, admissible & ~forced, chosen, cum, k_more, lane, [&](uint64_t, int n) { return n >= k_more; });
     result = chosen;
   }
   write_row<KPL>(result, p.idx + row * p.cap, p.cap, p.counts + row, lane);
