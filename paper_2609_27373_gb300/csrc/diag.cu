@@ -10,6 +10,19 @@
 namespace wise {
 namespace {
 
+// The row of query head bh and query block q of a support list.  Rows are
+// divided in 32 bits (those of a launch, n_blocks masses each and n_blocks to a
+// head, do not reach 2^32 in any memory); 64-bit division was half of the time
+// of a row of eight entries.
+struct MassRow {
+  int q;
+  long long support;  // row of the support lists: heads lie in whole groups, so bh / group counts (b, kv head)
+};
+__device__ __forceinline__ MassRow mass_row(const SupportMassParams& p, uint32_t row) {
+  const uint32_t bh = row / (uint32_t)p.n_blocks;
+  return {(int)(row - bh * (uint32_t)p.n_blocks), (long long)(bh / (uint32_t)p.group) * p.n_blocks + row - bh * (uint32_t)p.n_blocks};
+}
+
 // Eight lanes per query-head row (b, h, q): the row's masses r_qb summed over
 // the key blocks of its kv-group's support list, in list order.  Entries that
 // are negative, beyond the query block, or not strictly above the previous
@@ -17,18 +30,14 @@ namespace {
 // Latency-bound: one lane per row took two dependent loads per entry; here
 // eight entries, and then their masses, are loaded at once, a prefix maximum
 // over the eight decides which entries count, and the sum still adds them one
-// after the other (4K, 32 heads, 8 entries: 3.3 us, here 1.9).
+// after the other (4K, 32 heads, 8 entries: 3.5 us, here 1.9).
 __global__ void __launch_bounds__(256) support_mass_kernel(const SupportMassParams p) {
   constexpr int kLanes = 8;
   const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
   if (row >= p.rows) return;  // for all lanes of a row
   const int lane = threadIdx.x % kLanes;
   const unsigned mask = 0xFFu << (threadIdx.x & 31 & ~(kLanes - 1));
-  const int q = (int)(row % p.n_blocks);
-  const long long bh = row / p.n_blocks;
-  const int h = (int)(bh % p.n_heads);
-  const int b = (int)(bh / p.n_heads);
-  const long long srow = ((long long)b * p.n_kv_heads + h / p.group) * p.n_blocks + q;
+  const auto [q, srow] = mass_row(p, (uint32_t)row);
   const int32_t* list = p.idx + srow * p.cap;
   const float* m = p.blockmass + row * p.n_blocks;
   int n = __ldg(p.counts + srow);
@@ -61,6 +70,35 @@ __global__ void __launch_bounds__(256) support_mass_kernel(const SupportMassPara
     v = next;
   }
   if (lane == 0) p.retained[row] = acc;
+  if (bad) atomicOr(p.status, kStatusBadSupport);
+}
+
+// One lane per row, for many rows: bound by their loads then, not by one row's
+// chain of them.
+__global__ void __launch_bounds__(256) support_mass_rows_kernel(const SupportMassParams p) {
+  const uint32_t row = blockIdx.x * blockDim.x + threadIdx.x;
+  if (row >= p.rows) return;
+  const auto [q, srow] = mass_row(p, row);
+  int n = __ldg(p.counts + srow);
+  int bad = 0;
+  if (n < 0 || n > p.cap) {
+    bad = 1;
+    n = n < 0 ? 0 : p.cap;
+  }
+  const int32_t* list = p.idx + srow * p.cap;
+  const float* m = p.blockmass + (long long)row * p.n_blocks;
+  float acc = 0.0f;
+  int prev = -1;
+  for (int i = 0; i < n; ++i) {
+    const int v = __ldg(list + i);
+    if (v >= 0 && v <= q && v > prev) {
+      acc += __ldg(m + v);
+      prev = v;
+    } else {
+      bad = 1;
+    }
+  }
+  p.retained[row] = acc;
   if (bad) atomicOr(p.status, kStatusBadSupport);
 }
 
@@ -298,6 +336,14 @@ cudaError_t launch_support_overlap(const SupportOverlapParams& p, cudaStream_t s
 }
 
 cudaError_t launch_support_mass(const SupportMassParams& p, cudaStream_t stream) {
+  // Many rows, of lists of up to 16 entries: one lane
+  // each (131072 rows of 12, lists of 2 / 8: 8.7 / 8.6 us with eight lanes and 64-bit
+  // division, 6.9 / 6.9 without, 3.3 / 5.0 with one; rows of 64, lists of 32: 13 with
+  // one, 7.6 with eight).
+  if (p.rows > 32768 && p.cap <= 16) {
+    support_mass_rows_kernel<<<(unsigned)((p.rows + 255) / 256), 256, 0, stream>>>(p);
+    return cudaGetLastError();
+  }
   const long long blocks = (p.rows * 8 + 255) / 256;
   support_mass_kernel<<<(unsigned)blocks, 256, 0, stream>>>(p);
   return cudaGetLastError();
