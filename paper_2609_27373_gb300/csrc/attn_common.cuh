@@ -203,7 +203,7 @@ __device__ __forceinline__ int clamp_count(int n, int cap, int& bad) {
 }
 
 template <int BLK, int MODE>
-__device__ __forceinline__ TileIter<BLK, MODE> make_iter(const AttnParams& p, int b, int kvh, int qt) {
+__device__ __forceinline__ TileIter<BLK, MODE> make_iter(const AttnCore& p, int b, int kvh, int qt) {
   TileIter<BLK, MODE> it;
   it.bad = 0;
   if constexpr (MODE != kSparse) {
@@ -234,7 +234,7 @@ __device__ __forceinline__ TileIter<BLK, MODE> make_iter(const AttnParams& p, in
 // groups of group_heads consecutive ones (whole kv-head groups), all units of
 // a group before the next, so that the K and V of a group stay in L2 while
 // all its query tiles read them.
-__device__ __forceinline__ void decode_unit(const AttnParams& p, int u, int& b, int& h, int& qt) {
+__device__ __forceinline__ void decode_unit(const AttnCore& p, int u, int& b, int& h, int& qt) {
   const int bh_count = p.batch * p.n_heads;
   int bh;
   if (p.group_heads > 0) {
@@ -258,7 +258,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, limit_ns));
 }
 
-__device__ __forceinline__ void raise_status(const AttnParams& p, int* abort, int bits) {
+__device__ __forceinline__ void raise_status(const AttnCore& p, int* abort, int bits) {
   *reinterpret_cast<volatile int*>(abort) = 1;
   atomicOr(p.status, bits);
 }

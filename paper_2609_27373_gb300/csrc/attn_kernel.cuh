@@ -77,6 +77,8 @@
 #include <limits.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "attn_common.cuh"
 #include "internal.cuh"
 #include "ptx.cuh"
@@ -139,7 +141,7 @@ constexpr int kStageKeys = 128;
 constexpr int kStageTiles = 256;
 constexpr int kStageSlots = 4;
 template <int BLK, int MODE>
-__device__ __forceinline__ bool sched_staging(const AttnParams& p) {
+__device__ __forceinline__ bool sched_staging(const AttnCore& p) {
   constexpr int S = kTileN / BLK;
   return MODE == kSparse && S > 1 && p.cap <= kStageKeys / S && p.n_qtiles <= kStageTiles;
 }
@@ -197,7 +199,7 @@ struct SharedState {
 // global load per list entry on a thread that shares its scheduler with two
 // busy softmax warps.
 template <int D, int BLK, int MODE>
-__device__ void attn_sched_stager(const AttnParams& p, SharedState<AttnCfg<D>::kRingK, AttnCfg<D>::kRingV>& sb) {
+__device__ void attn_sched_stager(const AttnCore& p, SharedState<AttnCfg<D>::kRingK, AttnCfg<D>::kRingV>& sb) {
   constexpr int S = kTileN / BLK;
   constexpr int kCap = kStageKeys / S;      // list positions staged per query block (>= cap)
   constexpr int kRegs = kStageKeys / 32;    // entry e = lane + 32 i in register i
@@ -282,7 +284,7 @@ __device__ void attn_sched_stager(const AttnParams& p, SharedState<AttnCfg<D>::k
 // ------------------------------------------------------------------ producer
 template <int D, int BLK, int MODE>
 __device__ void attn_producer(const CUtensorMap* mapQ, const CUtensorMap* mapK, const CUtensorMap* mapV,
-                              const AttnParams& p, uint8_t* q_stage, uint8_t* ring,
+                              const AttnCore& p, uint8_t* q_stage, uint8_t* ring,
                               SharedState<AttnCfg<D>::kRingK, AttnCfg<D>::kRingV>& sb) {
   using C = AttnCfg<D>;
   constexpr int RK = C::kRingK, RV = C::kRingV;
@@ -437,7 +439,7 @@ __device__ void attn_producer(const CUtensorMap* mapQ, const CUtensorMap* mapK, 
 
 // --------------------------------------------------------------- MMA issuers
 template <int D, int BLK, int MODE>
-__device__ void attn_mma_s(const AttnParams& p, uint32_t tmem, uint8_t* q_stage, uint8_t* ring,
+__device__ void attn_mma_s(const AttnCore& p, uint32_t tmem, uint8_t* q_stage, uint8_t* ring,
                            SharedState<AttnCfg<D>::kRingK, AttnCfg<D>::kRingV>& sb) {
   using C = AttnCfg<D>;
   constexpr int RK = C::kRingK;
@@ -501,7 +503,7 @@ __device__ void attn_mma_s(const AttnParams& p, uint32_t tmem, uint8_t* q_stage,
 }
 
 template <int D, int BLK, int MODE>
-__device__ void attn_mma_pv(const AttnParams& p, uint32_t tmem, uint8_t* ring,
+__device__ void attn_mma_pv(const AttnCore& p, uint32_t tmem, uint8_t* ring,
                             SharedState<AttnCfg<D>::kRingK, AttnCfg<D>::kRingV>& sb) {
   using C = AttnCfg<D>;
   constexpr int RK = C::kRingK, RV = C::kRingV;
@@ -568,7 +570,7 @@ struct EpiInfo {
 
 // ------------------------------------------------------------------- softmax
 template <int D, int BLK, int MODE>
-__device__ void attn_softmax(const AttnParams& p, int w, uint32_t tmem, uint8_t* out_stage,
+__device__ void attn_softmax(const AttnCore& p, int w, uint32_t tmem, uint8_t* out_stage,
                              float* mass_ws,
                              SharedState<AttnCfg<D>::kRingK, AttnCfg<D>::kRingV>& sb) {
   using C = AttnCfg<D>;
@@ -922,11 +924,21 @@ __device__ void attn_softmax(const AttnParams& p, int w, uint32_t tmem, uint8_t*
   if (!ok) raise_status(p, &sb.abort, kStatusTimeout);
 }
 
+// The parameters an instance is launched with.  Those of attn_duo_kernel make
+// the block longer than 128 bytes, and registers are then allocated in another
+// way: dense and mass 2 to 8 % faster (13 heads, 4K, dense + mass, d 96 55.0 -> 50.6 us,
+// d 128 54.9 -> 52.9; d 64 dense 44.1 -> 41.0), but at head dim 128 the block masses
+// of blocks below 128 no longer fit (80 bytes of stack; 83 heads, 512 tokens 15.5 ->
+// 18.6 us), and these keep the short block.
+template <int D, int BLK, int MODE>
+using AttnLaunchParams = std::conditional_t<D == 128 && BLK < 128 && MODE == kDenseMass, AttnCore, AttnParams>;
+static_assert(sizeof(AttnCore) <= 128 && sizeof(AttnParams) > 128, "see AttnLaunchParams");
+
 // -------------------------------------------------------------------- kernel
 template <int D, int BLK, int MODE>
 __global__ void __launch_bounds__(AttnCfg<D>::kThreads, 1)
     attn_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                const __grid_constant__ CUtensorMap mapV, const AttnParams p) {
+                const __grid_constant__ CUtensorMap mapV, const AttnLaunchParams<D, BLK, MODE> p) {
   using C = AttnCfg<D>;
   using SS = SharedState<C::kRingK, C::kRingV>;
   static_assert(sizeof(SS) <= C::kStaticReserve, "static shared memory");
@@ -1032,7 +1044,8 @@ __global__ void __launch_bounds__(AttnCfg<D>::kThreads, 1)
 template <int D, int BLK, int MODE>
 cudaError_t launch_attn_instance(const AttnLaunch& L) {
   using C = AttnCfg<D>;
-  return launch_dependent<attn_kernel<D, BLK, MODE>>(L.grid, C::kThreads, C::kSmemLaunch, L.stream, L.mapQ, L.mapK, L.mapV, L.p);
+  return launch_dependent<attn_kernel<D, BLK, MODE>>(L.grid, C::kThreads, C::kSmemLaunch, L.stream, L.mapQ, L.mapK,
+                                                     L.mapV, static_cast<const AttnLaunchParams<D, BLK, MODE>&>(L.p));
 }
 
 template <int D>

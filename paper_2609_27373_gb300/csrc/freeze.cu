@@ -37,7 +37,7 @@ struct FzCfg {
 };
 
 template <int BLK>
-__device__ __forceinline__ int walk_length(const AttnParams& p, int b, int kvh, int qt) {
+__device__ __forceinline__ int walk_length(const AttnCore& p, int b, int kvh, int qt) {
   auto it = make_iter<BLK, kSparse>(p, b, kvh, qt);
   int kt, n = 0;
   uint32_t mask;
@@ -64,7 +64,7 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 template <int D, int BLK>
 __global__ void __launch_bounds__(160, 1)
     freeze_probs_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                        const AttnParams p, __nv_bfloat16* P, float* inv_l, int tile_cap) {
+                        const AttnCore p, __nv_bfloat16* P, float* inv_l, int tile_cap) {
   using C = FzCfg<D>;
   constexpr int S = kTileN / BLK;
   extern __shared__ uint8_t smem_raw[];
@@ -245,7 +245,7 @@ struct PvShared {
 template <int D, int BLK>
 __global__ void __launch_bounds__(192, 1)
     frozen_pv_kernel(const __grid_constant__ CUtensorMap mapP, const __grid_constant__ CUtensorMap mapV,
-                     const AttnParams p, const float* inv_l, int tile_cap) {
+                     const AttnCore p, const float* inv_l, int tile_cap) {
   using C = FzCfg<D>;
   constexpr int kStage = C::kPBytes + C::kKBytes;
   extern __shared__ uint8_t smem_raw[];

@@ -30,7 +30,7 @@ constexpr int kStatusBadSupport = 2;
 // How the two streams of attn_duo_kernel take query tiles (attn_duo.cuh).
 enum AttnPair : int { kPairNone = 0, kPairHeads = 1, kPairTiles = 2 };
 
-struct AttnParams {
+struct AttnCore {
   int batch, seqlen, n_heads, n_kv_heads, group;
   int n_qtiles;   // ceil(seqlen / 128): 128-row query tiles
   int n_blocks;   // nQB = nKB = seqlen / block
@@ -46,6 +46,9 @@ struct AttnParams {
   float* scratch;         // kDenseMass: scratch_floats_per_cta(n_blocks) floats per CTA
   int* status;
   unsigned long long wait_ns;  // limit of each bounded wait on the main path (kWaitLimitNs by default)
+};
+
+struct AttnParams : AttnCore {
   // attn_duo_kernel: the pairing, and its units (virtual heads and query
   // tiles, see decode_duo).
   int pair, v_heads, v_qtiles, v_units, v_group_heads;
@@ -135,7 +138,7 @@ struct SupportMassParams {
 struct FreezeLaunch {
   CUtensorMap mapQ, mapK;  // wise_freeze_a_probs: the frozen step's Q and K (128-row boxes)
   CUtensorMap mapV, mapP;  // wise_frozen_pv: current V, and P viewed as [tiles][128][128]
-  AttnParams p;            // shape, support lists, scale, status; O for wise_frozen_pv
+  AttnCore p;              // shape, support lists, scale, status; O for wise_frozen_pv
   __nv_bfloat16* P;
   float* inv_l;
   int tile_cap;

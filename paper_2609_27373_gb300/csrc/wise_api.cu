@@ -340,7 +340,7 @@ int freeze_setup(const wise_shape_t* sh, const int32_t* idx, const int32_t* coun
   int err = WISE_OK;
   DeviceState* ds = device_state(&err);
   if (!ds) return err;
-  AttnParams& p = L.p;
+  AttnCore& p = L.p;
   memset(&p, 0, sizeof(p));
   p.batch = sh->batch;
   p.seqlen = sh->seqlen;
