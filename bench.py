@@ -58,14 +58,26 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 
 
+# What decides the sparse kernel's traffic: the kernel, what it includes, and its
+# boxes, pairing and grid.
+SPARSE_SOURCES = ("attn_duo.cuh", "attn_common.cuh", "ptx.cuh", "internal.cuh", "wise_api.cu")
+
+
+def sparse_sources_sha():
+    import hashlib
+    h = hashlib.sha256()
+    for name in SPARSE_SOURCES:
+        with open(os.path.join(ROOT, "paper_2609_27373_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def sparse_traffic_bytes():
     """DRAM bytes per launch of the sparse kernel from the committed ncu
-    summary, or None when the kernel source changed since that capture."""
-    import hashlib
-    src = os.path.join(ROOT, "paper_2609_27373_gb300", "csrc", "attn_duo.cuh")
+    summary, or None when a source it depends on changed since that capture."""
     prof = os.path.join(ROOT, "profiles", "attn_sparse_4k.md")
     try:
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+        sha = sparse_sources_sha()
         fields = dict(line.split(":", 1) for line in open(prof) if line.count(":") == 1 and " " not in line.split(":")[0])
     except (OSError, ValueError):
         return None
