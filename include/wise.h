@@ -33,7 +33,9 @@
  *    programmatic dependents: their set-up, and their reads of idx and counts,
  *    may overlap the end of the preceding attention call on the same stream,
  *    whose other effects they wait for.  So idx and counts must not share
- *    memory with the O or blockmass of the preceding attention call.
+ *    memory with the O or blockmass of the preceding attention call, nor be
+ *    written by a kernel right before the call that lets its dependents start
+ *    before it ends (a programmatic launch trigger of the caller's own).
  *  - Inputs are never written.  The library keeps one lazily allocated
  *    scratch buffer per device for the block-mass epilogue (see
  *    wise_full_attn_accumulate); no other call allocates device memory.

@@ -24,9 +24,16 @@
 // Tensor memory (512 columns): S of stream s at 128 s, with P (bf16 pairs)
 // written over its first 64 columns, and O of stream s at 256 + 128 s.
 // S(j+1) of a stream overwrites P(j), so it is issued right behind P V(j) by
-// the same thread: the tensor pipe runs one thread's products in order, and no
-// barrier is needed between them.  It also follows that S(j+1) complete means
-// P V(j) complete: the softmax may rescale O without a further wait, and the
+// the same thread, with no barrier between them.  This relies on the tensor
+// pipe running one thread's tcgen05.mma of one CTA group in the order of issue.
+// The ISA states that for products of the same shape and accumulator; these two
+// have different accumulators (and, at head dims 64 and 96, shapes), so here it
+// is the hardware's behaviour that is relied on, not a documented guarantee.
+// An S product that ran ahead would change P under P V: outputs that differ
+// between runs (the repeated launches of test_determinism_gpu.py) or from the
+// oracle (test_duo_gpu.py).  It also follows that S(j+1) complete means P V(j)
+// complete (a commit tracks all earlier products of its thread, which is
+// documented): the softmax may rescale O without a further wait, and the
 // epilogue's read of O precedes the next unit's first P V because the same
 // warpgroup writes that P.
 //
@@ -52,7 +59,10 @@
 // issuing warp sees P, P V and S(j+1) behind one another.  attn_kernel takes
 // 1930 clk a tile.  A unit boundary costs a sparse stream 4400 clk more (16K, 11
 // tiles a unit): the diagonal's mask 600-1000, O's last product and the
-// epilogue 3100, the rest of the wait for the next unit's Q and first S.
+// epilogue 3100, the rest of the wait for the next unit's Q and first S.  These
+// do not add up to an unpaired launch: 16K, 142 tiles and 13.5 units a stream in
+// 302 us, leaves 3660 clk a tile besides the boundaries (paired 32K 3130); the
+// likely part is the wait for V and K, whose buffers are one and a half tiles.
 // Measured against attn_kernel (us, before / here): dense 120 / 102, dense + mass
 // 130 / 111, sparse block 128 64 / 57, block 32 150 / 110; 16K sparse 352 / 286; 32K,
 // four heads to a kv head 855 / 690 (paired); 4 x 4K, head dim 96 405 / 298.

@@ -13,12 +13,14 @@ namespace wise {
 enum AttnMode : int { kDense = 0, kDenseMass = 1, kSparse = 2 };
 
 // Per-CTA scratch of kDenseMass, in floats, for n_tiles key tiles of 128
-// keys holding sub key blocks each (n_blocks key blocks in all): log2 partial
-// masses [2 warpgroups][2 units][n_tiles / 2 + 1][sub][128 rows] (a
+// keys holding sub key blocks each (n_blocks key blocks in all).  attn_kernel:
+// log2 partial masses [2 warpgroups][2 units][n_tiles / 2 + 1][sub][128 rows] (a
 // warpgroup handles every other tile of a unit, and keeps the previous unit's
 // values until its epilogue has read them), then per-warp column sums
 // [2 warpgroups][2][4 warps][n_blocks] (used only when the kernel's shared
 // memory copy of them, for up to 128 key blocks, is too small).
+// attn_duo_kernel uses the front of it: partial masses [2 streams][n_tiles][sub]
+// [128 rows] of the unit each stream works on.
 __host__ __device__ constexpr size_t scratch_floats_per_cta(int n_tiles, int sub, int n_blocks) {
   return (size_t)512 * sub * (n_tiles / 2 + 1) + (size_t)16 * n_blocks;
 }
@@ -43,7 +45,7 @@ struct AttnCore {
   const int32_t* idx;     // kSparse
   const int32_t* counts;  // kSparse
   int cap;                // kSparse
-  float* scratch;         // kDenseMass: scratch_floats_per_cta(n_blocks) floats per CTA
+  float* scratch;         // kDenseMass: scratch_floats_per_cta() floats per CTA
   int* status;
   unsigned long long wait_ns;  // limit of each bounded wait on the main path (kWaitLimitNs by default)
 };

@@ -2,11 +2,14 @@
 // loads, tcgen05 tensor-memory allocation, UMMA (tcgen05.mma kind::f16) with
 // shared-memory descriptors, and tcgen05 tensor-memory loads/stores.
 //
-// Layout conventions used by every kernel of this library:
+// Layout conventions used by the kernels of this library:
 //  * Operand tiles live in shared memory in the 128-byte-swizzle layout that
 //    a TMA box of 64 bf16 columns x R rows produces: row r of the box is 128
 //    bytes at offset r*128, and its 16-byte chunk c is stored at chunk
-//    position c ^ (r & 7).  Boxes are 1024-byte aligned.
+//    position c ^ (r & 7).  Boxes are 1024-byte aligned.  (Unpaired launches of
+//    attn_duo_kernel at head dim 96 use boxes of 32 columns in the 64-byte
+//    swizzle: rows of 64 bytes, chunk c at position c ^ ((r >> 1) & 3), K step kk
+//    in box kk/2.)
 //  * A K-major operand (rows x K) is a sequence of such boxes, one per 64
 //    K-columns; a 16-wide K step kk starts at box kk/4, byte (kk%4)*32.
 //  * An MN-major operand (K rows x N columns, N contiguous) is a sequence of

@@ -154,7 +154,9 @@ bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long
 // 1.00-1.11 / 1.15-1.28).  Not so with an odd number of query tiles, whose last
 // has no partner (dense, 384 tokens 0.86), 512 tokens at d 128 (dense 0.95), 1K
 // tokens (dense 0.79-0.91), or more than two units per SM (dense, 256 tokens
-// 0.85).
+// 0.85).  At the line itself sparse launches of d 128 lose a little (480 units: 4K,
+// 15 heads 29.8 / 31.7, 2K, 15 head pairs 27.1 / 28.3) where dense and mass ones gain
+// 12 to 23 %.
 // The line depends on the shape alone, not on the variant: sparse attention
 // over every block and dense attention run on the same kernel and give the
 // same bits.  One query tile is the exception: a unit of one key tile comes out
@@ -163,7 +165,9 @@ bool make_map(CUtensorMap* map, const void* base, int head_dim, int seqlen, long
 // 14.1 / 15.1, 17.5 / 19.4, 22.2 / 24.6; dense + mass 24.0 / 18.4, 26.7 / 19.1, 30.4 /
 // 26.0, sparse, unpaired, 17.0 / 13.9, 18.7 / 15.5, 23.6 / 21.4).
 bool choose_duo(int mode, int head_dim, int sm_count, AttnParams& p) {
-  if (p.n_qtiles > 256) return false;  // the staged tile masks hold 256 key tiles
+  // The staged tile masks of a sparse launch hold 256 key tiles; dense launches
+  // follow it, to agree with it bit for bit.
+  if (p.n_qtiles > 256) return false;
   const bool side_by_side = (p.n_qtiles == 2 || (p.n_qtiles == 4 && head_dim < 128)) &&
                             2 * (long long)p.n_units >= 3 * sm_count && p.n_units <= 2 * sm_count;
   if (p.n_units < 3 * sm_count && !side_by_side) return false;
