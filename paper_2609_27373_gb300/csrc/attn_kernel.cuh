@@ -94,8 +94,8 @@ struct AttnCfg {
   static constexpr int kStaticReserve = 10 * 1024;
   // Dynamic shared memory available after the 1024-byte alignment slack.
   static constexpr int kBudget = 227 * 1024 - 1024 - kStaticReserve;
-  // Epilogue staging: per softmax warp of L, 32 rows x 64 columns of O
-  // (one 128-byte-swizzled TMA box).
+  // Epilogue staging: per softmax warp of L, 32 rows x 64 columns of O (in the
+  // 128-byte swizzle).
   static constexpr int kOutBytes = 4 * 32 * 128;
   // Block-mass epilogue: per-warp column sums [2 buffers][4 warps][key
   // blocks] for up to kMassWsBlocks key blocks (more go to the global scratch).
